@@ -117,10 +117,6 @@ struct Plan {
   // backward
   long long group = 0, ngroups = 0;
   size_t off_invn = 0, off_G = 0, bwd_bytes = 0;
-  // fp32 inputs only: K-major copies G^T [M][group][t_pitch], H_m^T [d_m][t_pitch],
-  // W_m^T [d_m][v_pitch] for the tf32 GEMMs
-  long long t_pitch = 0, v_pitch = 0;
-  size_t off_GT = 0, off_HT[kMaxModels] = {}, off_WT[kMaxModels] = {};
   // pairwise evaluation
   int eval_nvt = 0, eval_S = 1;
   size_t off_epart = 0, off_eacc = 0, off_ecnt = 0, eval_bytes = 0;
@@ -240,18 +236,6 @@ Plan make_plan(const mls_problem* p, int pairs) {
   o = align_up(o + sizeof(float));
   pl.off_G = o;
   o = align_up(o + static_cast<size_t>(pl.elt) * M * T * pl.group);
-  if (pl.elt == 4) {
-    pl.t_pitch = ceil_div(T, 4) * 4;
-    pl.v_pitch = ceil_div(V, 4) * 4;
-    pl.off_GT = o;
-    o = align_up(o + sizeof(float) * static_cast<size_t>(M) * pl.group * pl.t_pitch);
-    for (int m = 0; m < p->M; ++m) {
-      pl.off_HT[m] = o;
-      o = align_up(o + sizeof(float) * static_cast<size_t>(p->d[m]) * pl.t_pitch);
-      pl.off_WT[m] = o;
-      o = align_up(o + sizeof(float) * static_cast<size_t>(p->d[m]) * pl.v_pitch);
-    }
-  }
   pl.bwd_bytes = o;
 
   pl.eval_nvt = static_cast<int>(ceil_div(V, eval_tile_cols(p->M)));
@@ -514,40 +498,24 @@ extern "C" int mls_head_loss_bwd(const mls_problem* p, const void* const* H, con
   hp.g_pitch = pl.group;
   hp.g_model_stride = p->T * pl.group;
 
-  // bf16: dW reads A = G viewed M-major and B = H viewed N-major, dH reads
-  // A = G K-major and B = W viewed N-major, all in place.
-  // fp32 (tf32 MMA): dW reads A = G^T and B = H^T, dH reads A = G and B = W^T,
-  // all K-major.
+  // dW reads A = G viewed M-major and B = H viewed N-major, dH reads A = G
+  // K-major and B = W viewed N-major, all in place.
   GemmParams gw, gh, gb;
   std::memset(&gw, 0, sizeof gw);
   std::memset(&gh, 0, sizeof gh);
-  float* GT = tf32 ? reinterpret_cast<float*>(wsb + pl.off_GT) : nullptr;
+  const CUtensorMapSwizzle mn_swizzle =
+      tf32 ? CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B : CU_TENSOR_MAP_SWIZZLE_128B;
   for (int m = 0; m < p->M; ++m) {
     const void* Gm = static_cast<const char*>(G) + static_cast<size_t>(pl.elt) * hp.g_model_stride * m;
-    if (encode(&gh.mapA[m], Gm, pl.elt, pl.group, p->T, pl.group, KE, kGemmBM)) return MLS_ERR_CUDA;
     // the backward head kernel's TMA stores of 32x32 dL/dz chunks (bf16 only)
     if (!tf32 && encode(&hp.mapG[m], Gm, 2, pl.group, p->T, pl.group, 32, 32,
                         CU_TENSOR_MAP_SWIZZLE_64B))
       return MLS_ERR_CUDA;
-    if (!tf32) {
-      if (encode(&gw.mapA[m], Gm, pl.elt, pl.group, p->T, pl.group, KE, KE) ||
-          encode(&gw.mapB[m], H[m], pl.elt, p->d[m], p->T, p->d[m], KE, KE) ||
-          encode(&gh.mapB[m], W[m], pl.elt, p->d[m], p->V, p->d[m], KE, KE))
-        return MLS_ERR_CUDA;
-    } else {
-      float* HT = reinterpret_cast<float*>(wsb + pl.off_HT[m]);
-      float* WT = reinterpret_cast<float*>(wsb + pl.off_WT[m]);
-      if ((rc = launch_ok(launch_transpose(static_cast<const float*>(H[m]), p->T, p->d[m], p->d[m],
-                                           HT, pl.t_pitch, s))) ||
-          (rc = launch_ok(launch_transpose(static_cast<const float*>(W[m]), p->V, p->d[m], p->d[m],
-                                           WT, pl.v_pitch, s))))
-        return rc;
-      if (encode(&gw.mapA[m], GT + static_cast<size_t>(m) * pl.group * pl.t_pitch, 4, p->T,
-                 pl.group, pl.t_pitch, KE, kGemmBM) ||
-          encode(&gw.mapB[m], HT, 4, p->T, p->d[m], pl.t_pitch, KE, kGemmBHalf) ||
-          encode(&gh.mapB[m], WT, 4, p->V, p->d[m], pl.v_pitch, KE, kGemmBHalf))
-        return MLS_ERR_CUDA;
-    }
+    if (encode(&gh.mapA[m], Gm, pl.elt, pl.group, p->T, pl.group, KE, kGemmBM) ||
+        encode(&gw.mapA[m], Gm, pl.elt, pl.group, p->T, pl.group, KE, KE, mn_swizzle) ||
+        encode(&gw.mapB[m], H[m], pl.elt, p->d[m], p->T, p->d[m], KE, KE, mn_swizzle) ||
+        encode(&gh.mapB[m], W[m], pl.elt, p->d[m], p->V, p->d[m], KE, KE, mn_swizzle))
+      return MLS_ERR_CUDA;
   }
   gw.nprob = gh.nprob = p->M;
   gw.status = gh.status = dev->status;
@@ -562,14 +530,6 @@ extern "C" int mls_head_loss_bwd(const mls_problem* p, const void* const* H, con
     hp.band = pl.band_bwd;
     hp.g_col0 = c0;
     if ((rc = timed("head_bwd", s, [&] { return launch_head_bwd(hp, tf32, p->tau == 1.0f, s); }))) return rc;
-    if (tf32)
-      for (int m = 0; m < p->M; ++m)
-        if ((rc = launch_ok(launch_transpose(
-                 reinterpret_cast<const float*>(G) + static_cast<size_t>(m) * hp.g_model_stride,
-                 p->T, pl.group, pl.group, GT + static_cast<size_t>(m) * pl.group * pl.t_pitch,
-                 pl.t_pitch, s))))
-          return rc;
-
     int tw = 0, th = 0;
     for (int m = 0; m < p->M; ++m) {
       GemmProblem& a = gw.prob[m];
@@ -601,13 +561,7 @@ extern "C" int mls_head_loss_bwd(const mls_problem* p, const void* const* H, con
     gh.total_tiles = th;
     // persistent: one CTA pair per resident pair slot, never more pairs than tiles
     const int pairs = dev->gemm_pairs;
-    const int grid_w = 2 * (tw < pairs ? tw : pairs), grid_h = 2 * (th < pairs ? th : pairs);
-    if (tf32) {
-      if ((rc = timed("gemm_dw", s, [&] { return launch_gemm_kk(gw, true, grid_w, s); }))) return rc;
-      if ((rc = timed("gemm_dh", s, [&] { return launch_gemm_kk(gh, true, grid_h, s); }))) return rc;
-      continue;
-    }
-    // bf16: dW and dH of every sub-model in one persistent launch, the class
+    // dW and dH of every sub-model in one persistent launch, the class
     // with the longer reduction (dH: the group's columns, dW: T) scheduled first.
     const bool dh_long = gc >= p->T;
     const GemmParams& L = dh_long ? gh : gw;
@@ -653,7 +607,7 @@ extern "C" int mls_head_loss_bwd(const mls_problem* p, const void* const* H, con
     const long long cost_l = (ceil_div(gb.prob[0].K, KE) + kDrainBlocks) * (gb.prob[0].wide ? 2 : 1);
     const long long cost_s = (ceil_div(gb.prob[M].K, KE) + kDrainBlocks) * (gb.prob[M].wide ? 2 : 1);
     schedule_two_class(gb, grid / 2, n_long, cost_l, units - n_long, cost_s);
-    if ((rc = timed("gemm_bwd", s, [&] { return launch_gemm_mixed(gb, grid, s); }))) return rc;
+    if ((rc = timed("gemm_bwd", s, [&] { return launch_gemm_mixed(gb, tf32, grid, s); }))) return rc;
   }
   return MLS_OK;
 }

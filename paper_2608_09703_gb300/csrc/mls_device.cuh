@@ -398,6 +398,29 @@ __device__ __forceinline__ uint64_t make_sdesc(uint32_t saddr, uint32_t lbo_byte
   return d;
 }
 
+// Descriptor of an MN-major operand of 32-bit elements (tf32): 128-byte swizzle
+// of 32-byte pieces (the layout TMA writes with
+// CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B), the only swizzled layout in which the
+// tf32 MMA reads transposed operands.  Rows of 128 bytes run along M/N, atoms
+// are 4 K rows (512 bytes, SBO), LBO as above; swizzle mode 1.
+__device__ __forceinline__ uint64_t make_sdesc_mn32(uint32_t saddr, uint32_t lbo_bytes) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
+  d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16;
+  d |= (uint64_t)(512u >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)1 << 61;
+  return d;
+}
+
+// An operand's descriptor by its layout: K-major, or MN-major with blocks of
+// `box` bytes (128 bytes of M/N by the K rows of one stage).
+template <bool kTF32>
+__device__ __forceinline__ uint64_t operand_desc(uint32_t saddr, bool mn, uint32_t box) {
+  if (!mn) return make_sdesc(saddr, 16u);
+  return kTF32 ? make_sdesc_mn32(saddr, box) : make_sdesc(saddr, box);
+}
+
 // 32 consecutive TMEM columns of this thread's lane (32x32b shape), waited on
 // inside the same asm block so the registers are valid when it returns.  The
 // whole warp must execute it together (.sync.aligned), hence the __syncwarp.

@@ -2,11 +2,14 @@
 //   dW_m[v, :] = sum_t G_m[t, v] H_m[t, :]     A = G_m viewed M-major (M = v), B = H_m N-major
 //   dH_m[t, :] = sum_v G_m[t, v] W_m[v, :]     A = G_m K-major (K = v),       B = W_m N-major
 // where G_m = dL/dz_m is the bf16 (fp32 for fp32 inputs) gradient tile written
-// by the backward head kernel.  For bf16 both products read the row-major
-// tensors in place: the shared-memory descriptors say which dimension is
-// contiguous, so no transposed copy of G, H or W is made.  The tf32 MMA is
-// only used with K-major operands here, so fp32 inputs go through transposed
-// copies (G^T, H^T, W^T) instead.
+// by the backward head kernel.  Both products read the row-major tensors in
+// place: the shared-memory descriptors say which dimension is contiguous, so
+// no transposed copy of G, H or W is made.  The tf32 MMA reads transposed
+// operands only in the 128-byte swizzle of 32-byte pieces, so the tensor maps
+// of fp32 MN-major operands use that one (operand_desc).  Transposed copies of
+// G, H and W took 1952 us for an fp32 step of 2048 tokens, d = (768, 1536),
+// V = 32768, and 110 us for 256 tokens, d = (128, 256), V = 1024; reading in
+// place takes 1635 and 74 us, with bit-identical gradients.
 //
 // CTA pairs (clusters of 2) own 256x256 output tiles: each CTA loads the 128
 // rows of A and the 128 rows of B that are its half, the even CTA issues
@@ -266,14 +269,14 @@ __device__ __forceinline__ void gemm_mma(const GemmParams& p, uint32_t base, uin
       tc_fence_after();
       const uint32_t sa = wide ? base + wstage * GemmSmem::kWideStage : base + GemmSmem::kA + stage * kGemmABytes;
       const uint32_t sb = wide ? sa + kGemmABytes : base + GemmSmem::kB + stage * kGemmBBytes;
-      const uint64_t ad = make_sdesc(sa, amn ? kBox : 16u);
-      const uint64_t bd = make_sdesc(sb, kBMN ? kBox : 16u);
+      const uint64_t ad = operand_desc<kTF32>(sa, amn, kBox);
+      const uint64_t bd = operand_desc<kTF32>(sb, kBMN, kBox);
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk)
         mma_issue_pair<kTF32>(d0, ad + kk * (amn ? kStepMN : kStepK),
                               bd + kk * (kBMN ? kStepMN : kStepK), idesc, (kb | kk) != 0);
       if (uc.nt == 2) {
-        const uint64_t bd1 = make_sdesc(sb + kGemmBBytes, kBMN ? kBox : 16u);  // second column tile
+        const uint64_t bd1 = operand_desc<kTF32>(sb + kGemmBBytes, kBMN, kBox);  // second column tile
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
           mma_issue_pair<kTF32>(d1, ad + kk * (amn ? kStepMN : kStepK),
@@ -559,16 +562,11 @@ cudaError_t launch(const GemmParams& p, bool tf32, int grid, cudaStream_t s) {
 
 }  // namespace
 
-cudaError_t launch_gemm_kk(const GemmParams& p, bool tf32, int grid, cudaStream_t s) {
-  return launch<0, false, false>(p, tf32, grid, s);
-}
 cudaError_t launch_gemm_stats(const GemmParams& p, bool tf32, int grid, cudaStream_t s) {
   return launch<0, false, true>(p, tf32, grid, s);
 }
-cudaError_t launch_gemm_mixed(const GemmParams& p, int grid, cudaStream_t s) {
-  if (p.total_tiles <= 0 || grid <= 0) return cudaSuccess;
-  gemm_kernel<false, 2, true, false><<<grid, kGemmThreads, kGemmSmem, s>>>(p);
-  return cudaGetLastError();
+cudaError_t launch_gemm_mixed(const GemmParams& p, bool tf32, int grid, cudaStream_t s) {
+  return launch<2, true, false>(p, tf32, grid, s);
 }
 
 // How many CTA pairs of the GEMM kernel can be resident at once (GPCs with an
@@ -598,10 +596,9 @@ cudaError_t setup_gemm_kernels() {
     if (e != cudaSuccess) return e;                                                             \
     if (fa.maxThreadsPerBlock < kGemmThreads) return cudaErrorLaunchOutOfResources;             \
   }
-  MLS_SET(true, 0, false, false)
-  MLS_SET(false, 0, false, false)
   MLS_SET(true, 0, false, true)
   MLS_SET(false, 0, false, true)
+  MLS_SET(true, 2, true, false)
   MLS_SET(false, 2, true, false)
 #undef MLS_SET
   return cudaSuccess;

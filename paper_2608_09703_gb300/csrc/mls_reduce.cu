@@ -1,5 +1,4 @@
-// Row reductions of the forward pass, the token count of the backward and an
-// fp32 transpose (used only for fp32 inputs, whose tf32 GEMMs read K-major copies).
+// Row reductions of the forward pass and the token count of the backward.
 //
 // merge_kernel: a block of 8 warps combines, for 8 to 64 tokens, the partial row
 // states that the head kernel wrote per (CTA, half tile) into
@@ -289,35 +288,7 @@ __global__ void __launch_bounds__(kCountThreads)
   if (threadIdx.x == 0) *inv_n = C > 0.0 ? static_cast<float>(1.0 / C) : 0.f;
 }
 
-// out[c][r] = in[r][c] for an fp32 [rows, cols] matrix, through 32x32 tiles.
-constexpr int kTile = 32;
-__global__ void __launch_bounds__(kTile * 8)
-    transpose_kernel(const float* __restrict__ in, long long rows, long long cols, long long ld_in,
-                     float* __restrict__ out, long long ld_out) {
-  __shared__ float tile[kTile][kTile + 1];
-  const long long r0 = static_cast<long long>(blockIdx.y) * kTile;
-  const long long c0 = static_cast<long long>(blockIdx.x) * kTile;
-  for (int i = threadIdx.y; i < kTile; i += blockDim.y) {
-    const long long r = r0 + i, c = c0 + threadIdx.x;
-    tile[i][threadIdx.x] = (r < rows && c < cols) ? in[r * ld_in + c] : 0.f;
-  }
-  __syncthreads();
-  for (int i = threadIdx.y; i < kTile; i += blockDim.y) {
-    const long long c = c0 + i, r = r0 + threadIdx.x;
-    if (c < cols && r < rows) out[c * ld_out + r] = tile[threadIdx.x][i];
-  }
-}
-
 }  // namespace
-
-cudaError_t launch_transpose(const float* in, long long rows, long long cols, long long ld_in,
-                             float* out, long long ld_out, cudaStream_t s) {
-  if (rows <= 0 || cols <= 0) return cudaSuccess;
-  const dim3 grid(static_cast<unsigned>((cols + kTile - 1) / kTile),
-                  static_cast<unsigned>((rows + kTile - 1) / kTile));
-  transpose_kernel<<<grid, dim3(kTile, 8), 0, s>>>(in, rows, cols, ld_in, out, ld_out);
-  return cudaGetLastError();
-}
 
 cudaError_t launch_merge(const MergeParams& p, int blocks, cudaStream_t s) {
   if (blocks <= 0) return cudaSuccess;
