@@ -92,13 +92,17 @@ int device_state(DeviceState** out) {
   return s.err;
 }
 
-// Co-resident head-kernel CTA pairs on the current device, for sizing a plan
-// without launching (76 on a GB300 when no device can be queried).
-int current_head_pairs() {
+// Co-resident CTA pairs of the head and GEMM kernels on the current device, for
+// sizing a plan without launching (76 on a GB300 when no device can be queried).
+void current_pairs(int& head, int& gemm) {
   DeviceState* dev = nullptr;
-  if (device_state(&dev) == MLS_OK && dev->head_pairs > 0) return dev->head_pairs;
+  head = gemm = 76;
+  if (device_state(&dev) == MLS_OK && dev->head_pairs > 0) {
+    head = dev->head_pairs;
+    gemm = dev->gemm_pairs;
+    return;
+  }
   cudaGetLastError();
-  return 76;
 }
 
 // ------------------------------------------------------------------ planning
@@ -116,7 +120,7 @@ struct Plan {
   size_t off_part = 0, off_bsum = 0, off_bcnt = 0, fwd_bytes = 0;
   // backward
   long long group = 0, ngroups = 0;
-  size_t off_invn = 0, off_G = 0, bwd_bytes = 0;
+  size_t off_invn = 0, off_G = 0, off_split = 0, bwd_bytes = 0;
   // pairwise evaluation
   int eval_nvt = 0, eval_S = 1;
   size_t off_epart = 0, off_eacc = 0, off_ecnt = 0, eval_bytes = 0;
@@ -173,6 +177,127 @@ int choose_band(int ntt, long long h_bytes_per_tile, long long budget) {
   return static_cast<int>((ntt + nbands - 1) / nbands);
 }
 
+// The dH problems of a backward GEMM launch run in wide units
+// (GemmProblem::wide) when each of them has a reduction of at least this many
+// k-blocks of 128 bytes, an even number of column tiles (no single-tile
+// units, which would only lose the epilogue overlap) and nothing to
+// accumulate (the first vocabulary group): a wide unit's two accumulators are
+// drained while no MMA runs, which costs a share inversely proportional to
+// the reduction and doubles when dH is read back.  Measured on one GB300 in a
+// seconds-long loop under the power cap: the 3-level suite at T = 8192 (786
+// k-blocks) gains 2.6% on the GEMM, while the paper's 3B suite (9 and 17
+// column tiles) lost 5% and the 4-level suite (504 k-blocks, four groups)
+// 2% when they ran wide.
+constexpr long long kWideMinBlocks = 512;
+
+// Cost of a unit beyond its k-blocks, in k-blocks: draining its 256x256 accumulator.
+constexpr long long kDrainBlocks = 8;
+
+// Short units that a pair left one long unit short takes first (two-class schedule).
+int catchup_units(int pairs, int n_long, long long cost_long, int n_short, long long cost_short) {
+  const int r = n_long % pairs;
+  if (r == 0) return 0;
+  const int c = static_cast<int>((cost_long + cost_short / 2) / cost_short);
+  const int most = n_short / (pairs - r);
+  return c < most ? c : most;
+}
+
+// Two-class schedule of a persistent GEMM launch whose first n_long tiles take
+// cost_long and the other n_short cost_short (K-blocks plus a per-tile
+// allowance): see GemmParams.  The pairs that get one long tile fewer take
+// `catchup` short tiles first, about the cost of that long tile.
+void schedule_two_class(GemmParams& g, int pairs, int n_long, long long cost_long, int n_short,
+                        long long cost_short) {
+  g.two_class = 0;
+  if (pairs < 1 || n_long <= 0 || n_short <= 0) return;
+  g.two_class = 1;
+  g.n_long = n_long;
+  g.catchup = catchup_units(pairs, n_long, cost_long, n_short, cost_short);
+}
+
+// Time of that schedule in k-blocks: the busiest pair.
+long long two_class_time(int pairs, int n_long, long long cost_long, int n_short, long long cost_short) {
+  const int r = n_long % pairs, q = n_long / pairs;
+  const int c = n_short > 0 ? catchup_units(pairs, n_long, cost_long, n_short, cost_short) : 0;
+  const int rest = n_short - c * (pairs - r);
+  auto share = [&](int first) { return static_cast<long long>(rest > first ? (rest - first + pairs - 1) / pairs : 0); };
+  const long long extra = r > 0 ? (q + 1) * cost_long + share(0) * cost_short : 0;
+  const long long plain = q * cost_long + (c + share(r)) * cost_short;
+  return extra > plain ? extra : plain;
+}
+
+// How one vocabulary group's dW + dH launch is cut: which class has the longer
+// reduction, whether dH runs in wide units, and into how many units the long
+// reductions are split (GemmProblem::ksplit).
+struct GemmCut {
+  bool dh_long = true, wide = false;
+  int ksplit = 1, kb_split = 0;
+  long long cost_long = 0, cost_short = 0;
+  long long part_floats = 0;  // workspace of the splits' copies
+};
+
+// With few output tiles the long reductions bound the launch.  Splitting each
+// over several units (at least kSplitMinBlocks each) costs one more pass over
+// the output per split and a launch to add them up: kSplitLaunch k-blocks (of
+// about 0.33 us) and one per kSplitBytes written and read.  A split has to be
+// estimated kSplitGain faster, so that large launches stay whole.  Measured,
+// launch whole against split with its sum: 300 tokens, d = (96, 400), V = 30000
+// in fp32 (6 dH tiles of 938 k-blocks) 261 against 84 us; 100 tokens, d =
+// (512, 1024), V = 20000 (6 of 313) 117 against 87 us; 20000 tokens, d =
+// (512, 1024), V = 600 (dW, 18 of 313) 117 against 102 us; but 256 tokens, d =
+// (128, 256), V = 1024 in fp32 (2 of 32) 22 against 25 us.
+constexpr int kSplitMinBlocks = 12, kSplitMost = 32;
+constexpr long long kSplitLaunch = 16, kSplitBytes = 1700000;
+constexpr double kSplitGain = 0.95;
+
+GemmCut cut_gemm(int M, const int32_t* d, long long T, long long gc, bool first, int KE, int pairs) {
+  GemmCut c;
+  c.dh_long = gc >= T;
+  int t_dh = 0, t_dw = 0;  // 256 x kGemmBN output tiles
+  long long sum_d = 0;
+  c.wide = first && ceil_div(gc, KE) >= kWideMinBlocks;
+  for (int m = 0; m < M; ++m) {
+    const int tn = static_cast<int>(ceil_div(d[m], kGemmBN));
+    t_dh += static_cast<int>(ceil_div(T, 2 * kGemmBM)) * tn;
+    t_dw += static_cast<int>(ceil_div(gc, 2 * kGemmBM)) * tn;
+    sum_d += d[m];
+    c.wide = c.wide && tn % 2 == 0;
+  }
+  const long long kb_dh = ceil_div(gc, KE), kb_dw = ceil_div(T, KE);
+  const long long kb_long = c.dh_long ? kb_dh : kb_dw;
+  const int n_long = c.dh_long ? t_dh : t_dw, n_short = c.dh_long ? t_dw : t_dh;
+  c.cost_short = (c.dh_long ? kb_dw : kb_dh) + kDrainBlocks;
+  c.cost_long = kb_long + kDrainBlocks;
+  const int w_dh = c.wide ? 2 : 1;  // dH units of two tiles
+  if (!c.dh_long) c.cost_short *= w_dh;
+  else c.cost_long *= w_dh;
+  const long long whole =
+      two_class_time(pairs, c.dh_long ? n_long / w_dh : n_long, c.cost_long,
+                     c.dh_long ? n_short : n_short / w_dh, c.cost_short);
+  const long long rows = c.dh_long ? T : gc, out_bytes = 4 * rows * sum_d;
+  double best = kSplitGain * static_cast<double>(whole);
+  for (int s = 2; s <= kSplitMost; ++s) {
+    const long long per = ceil_div(kb_long, s);
+    if (per < kSplitMinBlocks) break;
+    if ((s - 1) * per >= kb_long) continue;
+    const long long cost_short = (c.dh_long ? kb_dw : kb_dh) + kDrainBlocks;
+    const long long t = two_class_time(pairs, n_long * s, per + kDrainBlocks, n_short, cost_short) +
+                        kSplitLaunch + (s + 1) * out_bytes / kSplitBytes;
+    if (static_cast<double>(t) < best) {
+      best = static_cast<double>(t);
+      c.ksplit = s;
+      c.kb_split = static_cast<int>(per);
+    }
+  }
+  if (c.ksplit > 1) {
+    c.wide = false;
+    c.cost_long = c.kb_split + kDrainBlocks;
+    c.cost_short = (c.dh_long ? kb_dw : kb_dh) + kDrainBlocks;
+    c.part_floats = c.ksplit * rows * sum_d;
+  }
+  return c;
+}
+
 int validate(const mls_problem* p) {
   if (!p || p->M < 1 || p->M > MLS_MAX_MODELS || p->T < 0 || p->V < 1 || p->V > INT_MAX ||
       p->T > INT_MAX || !p->d)
@@ -193,7 +318,7 @@ int validate(const mls_problem* p) {
   return MLS_OK;
 }
 
-Plan make_plan(const mls_problem* p, int pairs) {
+Plan make_plan(const mls_problem* p, int pairs, int gemm_pairs) {
   Plan pl;
   pl.elt = p->in_dtype == MLS_BF16 ? 2 : 4;
   const long long T = p->T, V = p->V, M = p->M;
@@ -236,6 +361,19 @@ Plan make_plan(const mls_problem* p, int pairs) {
   o = align_up(o + sizeof(float));
   pl.off_G = o;
   o = align_up(o + static_cast<size_t>(pl.elt) * M * T * pl.group);
+  // copies of a split reduction's output: the full groups' or the last one's
+  pl.off_split = o;
+  if (T > 0) {
+    const long long last = V - (pl.ngroups - 1) * pl.group;
+    long long most = 0;
+    for (const long long g : {0LL, 1LL, pl.ngroups - 1}) {
+      if (g >= pl.ngroups) continue;
+      const GemmCut c = cut_gemm(p->M, p->d, T, g + 1 < pl.ngroups ? pl.group : last, g == 0,
+                                 128 / pl.elt, gemm_pairs);
+      if (c.part_floats > most) most = c.part_floats;
+    }
+    o = align_up(o + sizeof(float) * static_cast<size_t>(most));
+  }
   pl.bwd_bytes = o;
 
   pl.eval_nvt = static_cast<int>(ceil_div(V, eval_tile_cols(p->M)));
@@ -363,7 +501,9 @@ using namespace mls;
 
 extern "C" size_t mls_workspace_size(const mls_problem* p) {
   if (validate(p) != MLS_OK) return 0;
-  return make_plan(p, current_head_pairs()).total;
+  int head = 0, gemm = 0;
+  current_pairs(head, gemm);
+  return make_plan(p, head, gemm).total;
 }
 
 extern "C" int mls_head_loss_fwd(const mls_problem* p, const void* const* H, const void* const* W,
@@ -379,7 +519,7 @@ extern "C" int mls_head_loss_fwd(const mls_problem* p, const void* const* H, con
   }
   DeviceState* dev = nullptr;
   if ((rc = device_state(&dev))) return rc;
-  const Plan pl = make_plan(p, dev->head_pairs);
+  const Plan pl = make_plan(p, dev->head_pairs, dev->gemm_pairs);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (p->T == 0) return launch_ok(cudaMemsetAsync(loss, 0, sizeof(float), s));
   if ((rc = check_ws(pl, ws, ws_bytes, pl.total))) return rc;
@@ -421,39 +561,6 @@ extern "C" int mls_head_loss_fwd(const mls_problem* p, const void* const* H, con
   return timed("final", s, [&] { return launch_final(mp.block_sum, mp.block_cnt, pl.merge_blocks, loss, s); });
 }
 
-// The dH problems of a backward GEMM launch run in wide units
-// (GemmProblem::wide) when each of them has a reduction of at least this many
-// k-blocks of 128 bytes, an even number of column tiles (no single-tile
-// units, which would only lose the epilogue overlap) and nothing to
-// accumulate (the first vocabulary group): a wide unit's two accumulators are
-// drained while no MMA runs, which costs a share inversely proportional to
-// the reduction and doubles when dH is read back.  Measured on one GB300 in a
-// seconds-long loop under the power cap: the 3-level suite at T = 8192 (786
-// k-blocks) gains 2.6% on the GEMM, while the paper's 3B suite (9 and 17
-// column tiles) lost 5% and the 4-level suite (504 k-blocks, four groups)
-// 2% when they ran wide.
-constexpr long long kWideMinBlocks = 512;
-
-// Two-class schedule of a persistent GEMM launch whose first n_long tiles take
-// cost_long and the other n_short cost_short (K-blocks plus a per-tile
-// allowance): see GemmParams.  The pairs that get one long tile fewer take
-// `catchup` short tiles first, about the cost of that long tile.
-void schedule_two_class(GemmParams& g, int pairs, int n_long, long long cost_long, int n_short,
-                        long long cost_short) {
-  g.two_class = 0;
-  if (pairs < 1 || n_long <= 0 || n_short <= 0) return;
-  g.two_class = 1;
-  g.n_long = n_long;
-  const int r = n_long % pairs;
-  int catchup = 0;
-  if (r > 0) {
-    catchup = static_cast<int>((cost_long + cost_short / 2) / cost_short);
-    const int most = n_short / (pairs - r);
-    if (catchup > most) catchup = most;
-  }
-  g.catchup = catchup;
-}
-
 extern "C" int mls_head_loss_bwd(const mls_problem* p, const void* const* H, const void* const* W,
                                  const int32_t* targets, const float* stats, float grad_scale,
                                  float* const* dH, float* const* dW, void* ws, size_t ws_bytes,
@@ -469,7 +576,7 @@ extern "C" int mls_head_loss_bwd(const mls_problem* p, const void* const* H, con
   }
   DeviceState* dev = nullptr;
   if ((rc = device_state(&dev))) return rc;
-  const Plan pl = make_plan(p, dev->head_pairs);
+  const Plan pl = make_plan(p, dev->head_pairs, dev->gemm_pairs);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (p->T == 0) {
     for (int m = 0; m < p->M; ++m)
@@ -517,8 +624,6 @@ extern "C" int mls_head_loss_bwd(const mls_problem* p, const void* const* H, con
         encode(&gh.mapB[m], W[m], pl.elt, p->d[m], p->V, p->d[m], KE, KE, mn_swizzle))
       return MLS_ERR_CUDA;
   }
-  gw.nprob = gh.nprob = p->M;
-  gw.status = gh.status = dev->status;
 
   const long long tiles_per_group = pl.group / kHeadBN;
   for (long long g = 0; g < pl.ngroups; ++g) {
@@ -530,84 +635,63 @@ extern "C" int mls_head_loss_bwd(const mls_problem* p, const void* const* H, con
     hp.band = pl.band_bwd;
     hp.g_col0 = c0;
     if ((rc = timed("head_bwd", s, [&] { return launch_head_bwd(hp, tf32, p->tau == 1.0f, s); }))) return rc;
-    int tw = 0, th = 0;
-    for (int m = 0; m < p->M; ++m) {
-      GemmProblem& a = gw.prob[m];
-      a.Mrows = static_cast<int>(gc);
-      a.Ncols = p->d[m];
-      a.K = static_cast<int>(p->T);
-      a.a_map = a.b_map = m;
-      a.C = dW[m] + c0 * p->d[m];
-      a.ldc = p->d[m];
-      a.accumulate = 0;
-      a.tiles_n = static_cast<int>(ceil_div(p->d[m], kGemmBN));
-      a.tile_begin = tw;
-      tw += static_cast<int>(ceil_div(gc, 2 * kGemmBM)) * a.tiles_n;
-
-      GemmProblem& b = gh.prob[m];
-      b.Mrows = static_cast<int>(p->T);
-      b.Ncols = p->d[m];
-      b.K = static_cast<int>(gc);
-      b.a_map = b.b_map = m;
-      b.b_k0 = static_cast<int>(c0);
-      b.C = dH[m];
-      b.ldc = p->d[m];
-      b.accumulate = g > 0 ? 1 : 0;
-      b.tiles_n = static_cast<int>(ceil_div(p->d[m], kGemmBN));
-      b.tile_begin = th;
-      th += static_cast<int>(ceil_div(p->T, 2 * kGemmBM)) * b.tiles_n;
-    }
-    gw.total_tiles = tw;
-    gh.total_tiles = th;
-    // persistent: one CTA pair per resident pair slot, never more pairs than tiles
-    const int pairs = dev->gemm_pairs;
-    // dW and dH of every sub-model in one persistent launch, the class
-    // with the longer reduction (dH: the group's columns, dW: T) scheduled first.
-    const bool dh_long = gc >= p->T;
-    const GemmParams& L = dh_long ? gh : gw;
-    const GemmParams& S = dh_long ? gw : gh;
+    // dW and dH of every sub-model in one persistent launch, the class with the
+    // longer reduction (dH: the group's columns, dW: T) first.
+    const int pairs = dev->gemm_pairs, M = p->M;
+    const GemmCut cut = cut_gemm(M, p->d, p->T, gc, g == 0, KE, pairs);
+    float* split_ws = reinterpret_cast<float*>(wsb + pl.off_split);
+    SplitSumParams sum;
+    std::memset(&sum, 0, sizeof sum);
     std::memset(&gb, 0, sizeof gb);
-    const int M = p->M;
-    for (int m = 0; m < M; ++m) {
-      gb.mapA[m] = L.mapA[m];
-      gb.mapB[m] = L.mapB[m];
-      gb.prob[m] = L.prob[m];
-      gb.prob[m].a_map = gb.prob[m].b_map = m;
-      gb.prob[m].a_mn = dh_long ? 0 : 1;
-      gb.mapA[M + m] = S.mapA[m];
-      gb.mapB[M + m] = S.mapB[m];
-      gb.prob[M + m] = S.prob[m];
-      gb.prob[M + m].a_map = gb.prob[M + m].b_map = M + m;
-      gb.prob[M + m].a_mn = dh_long ? 1 : 0;
-    }
-    // dH with a long reduction runs in wide units (two column tiles sharing
-    // each A tile of G); the units are numbered problem by problem, the long
-    // class first.
-    bool wide = true;
-    for (int i = 0; i < 2 * M; ++i) {
-      const GemmProblem& q = gb.prob[i];
-      if (q.a_mn == 0)
-        wide = wide && q.accumulate == 0 && q.tiles_n % 2 == 0 && ceil_div(q.K, KE) >= kWideMinBlocks;
-    }
     int units = 0, n_long = 0;
+    long long split_off = 0;
     for (int i = 0; i < 2 * M; ++i) {
+      const int m = i % M;
+      const bool is_long = i < M, dh = is_long == cut.dh_long;
+      gb.mapA[i] = dh ? gh.mapA[m] : gw.mapA[m];
+      gb.mapB[i] = dh ? gh.mapB[m] : gw.mapB[m];
       GemmProblem& q = gb.prob[i];
-      q.wide = (wide && q.a_mn == 0) ? 1 : 0;
+      q.Mrows = static_cast<int>(dh ? p->T : gc);
+      q.Ncols = p->d[m];
+      q.K = static_cast<int>(dh ? gc : p->T);
+      q.a_map = q.b_map = i;
+      q.b_k0 = dh ? static_cast<int>(c0) : 0;
+      q.C = dh ? dH[m] : dW[m] + c0 * p->d[m];
+      q.ldc = p->d[m];
+      q.accumulate = dh && g > 0 ? 1 : 0;
+      q.a_mn = dh ? 0 : 1;
+      q.tiles_m = static_cast<int>(ceil_div(q.Mrows, 2 * kGemmBM));
+      q.tiles_n = static_cast<int>(ceil_div(p->d[m], kGemmBN));
+      q.wide = cut.wide && dh ? 1 : 0;
       q.tile_begin = units;
-      units += static_cast<int>(ceil_div(q.Mrows, 2 * kGemmBM)) * (q.wide ? (q.tiles_n + 1) / 2 : q.tiles_n);
+      units += q.tiles_m * (q.wide ? (q.tiles_n + 1) / 2 : q.tiles_n) * (is_long ? cut.ksplit : 1);
+      if (is_long && cut.ksplit > 1) {  // the units write their own sums, added up below
+        q.ksplit = cut.ksplit;
+        q.kb_split = cut.kb_split;
+        q.split_stride = cut.part_floats / cut.ksplit;
+        sum.out[m] = q.C;
+        sum.n4[m] = static_cast<long long>(q.Mrows) * p->d[m] / 4;
+        sum.accumulate = q.accumulate;
+        q.C = split_ws + split_off;
+        q.accumulate = 0;
+        sum.part[m] = q.C;
+        split_off += static_cast<long long>(q.Mrows) * p->d[m];
+      }
       if (i == M - 1) n_long = units;
     }
     gb.nprob = 2 * M;
     gb.total_tiles = units;
     gb.status = dev->status;
-    const int grid = 2 * (gb.total_tiles < pairs ? gb.total_tiles : pairs);
-    // cost of a unit: its K-blocks (twice for a wide one) plus an allowance for
-    // draining its 256x256 accumulators
-    constexpr long long kDrainBlocks = 8;
-    const long long cost_l = (ceil_div(gb.prob[0].K, KE) + kDrainBlocks) * (gb.prob[0].wide ? 2 : 1);
-    const long long cost_s = (ceil_div(gb.prob[M].K, KE) + kDrainBlocks) * (gb.prob[M].wide ? 2 : 1);
-    schedule_two_class(gb, grid / 2, n_long, cost_l, units - n_long, cost_s);
+    // persistent: one CTA pair per resident pair slot, never more pairs than units
+    const int grid = 2 * (units < pairs ? units : pairs);
+    schedule_two_class(gb, grid / 2, n_long, cut.cost_long, units - n_long, cut.cost_short);
     if ((rc = timed("gemm_bwd", s, [&] { return launch_gemm_mixed(gb, tf32, grid, s); }))) return rc;
+    if (cut.ksplit > 1) {
+      sum.nprob = M;
+      sum.nsplit = cut.ksplit;
+      sum.stride = cut.part_floats / cut.ksplit;
+      if ((rc = timed("split_sum", s, [&] { return launch_split_sum(sum, s); }))) return rc;
+    }
   }
   return MLS_OK;
 }
@@ -731,7 +815,7 @@ extern "C" int mls_head_loss_fwd_noalloc(const mls_problem* p, const void* const
   }
   DeviceState* dev = nullptr;
   if ((rc = device_state(&dev))) return rc;
-  const Plan pl = make_plan(p, dev->head_pairs);
+  const Plan pl = make_plan(p, dev->head_pairs, dev->gemm_pairs);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (p->T == 0) return launch_ok(cudaMemsetAsync(loss, 0, sizeof(float), s));
   if (pl.fwd_bytes > static_cast<size_t>(MLS_NOALLOC_SCRATCH_BYTES))
@@ -793,7 +877,7 @@ extern "C" int mls_head_pairwise(const mls_problem* p, const void* const* H, con
   }
   DeviceState* dev = nullptr;
   if ((rc = device_state(&dev))) return rc;
-  const Plan pl = make_plan(p, dev->head_pairs);
+  const Plan pl = make_plan(p, dev->head_pairs, dev->gemm_pairs);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (p->T == 0)
     return launch_ok(cudaMemsetAsync(pair_stats, 0, sizeof(float) * 2 * p->M * p->M, s));

@@ -78,6 +78,7 @@ constexpr int kPairM = 2 * kGemmBM;  // output rows of a pair tile
 
 struct UnitCoord {
   int prob, tm, tn, nt;  // problem, tile row, first tile column, tiles (1 or 2)
+  int ks;                // split of the reduction (0 unless GemmProblem::ksplit > 1)
 };
 
 // The j-th unit of this pair, or -1 when it has no more.
@@ -117,13 +118,31 @@ __device__ __forceinline__ UnitCoord decode_unit(const GemmParams& p, int u) {
   while (i + 1 < p.nprob && u >= p.prob[i + 1].tile_begin) ++i;
   const GemmProblem& pr = p.prob[i];
   const int local = u - pr.tile_begin;
-  if (pr.m_fast) return {i, local % pr.tiles_m, local / pr.tiles_m, 1};
+  if (pr.m_fast) return {i, local % pr.tiles_m, local / pr.tiles_m, 1, 0};
   if (wide_of<kAMode>(pr)) {
     const int un = (pr.tiles_n + 1) >> 1;
     const int tn = (local % un) * 2;
-    return {i, local / un, tn, pr.tiles_n - tn < 2 ? 1 : 2};
+    return {i, local / un, tn, pr.tiles_n - tn < 2 ? 1 : 2, 0};
   }
-  return {i, local / pr.tiles_n, local % pr.tiles_n, 1};
+  if (kAMode == 2 && pr.ksplit > 1) {
+    const int tiles = pr.tiles_m * pr.tiles_n, t = local % tiles;
+    return {i, t / pr.tiles_n, t % pr.tiles_n, 1, local / tiles};
+  }
+  return {i, local / pr.tiles_n, local % pr.tiles_n, 1, 0};
+}
+
+// The k-blocks [begin, end) that a unit reduces.
+template <bool kTF32>
+__device__ __forceinline__ void unit_kblocks(const GemmProblem& pr, const UnitCoord& uc, int& begin,
+                                             int& end) {
+  constexpr int KE = kTF32 ? 32 : 64;
+  const int nkb = (pr.K + KE - 1) / KE;
+  begin = 0;
+  end = nkb;
+  if (pr.ksplit > 1) {
+    begin = uc.ks * pr.kb_split;
+    end = min(nkb, begin + pr.kb_split);
+  }
 }
 
 // This CTA's loads: its 128 rows of A and its 128 rows of B (of both column
@@ -163,10 +182,11 @@ __device__ __forceinline__ void gemm_producer(const GemmParams& p, uint32_t base
     layout = wide ? 1 : 0;
     const CUtensorMap* ma = &p.mapA[pr.a_map];
     const CUtensorMap* mb = &p.mapB[pr.b_map];
-    const int nkb = (pr.K + KE - 1) / KE;
+    int kb_begin, kb_end;
+    unit_kblocks<kTF32>(pr, uc, kb_begin, kb_end);
     const int m0 = pr.a_m0 + uc.tm * kPairM + static_cast<int>(rank) * kGemmBM;
     const int n0 = pr.b_n0 + uc.tn * kGemmBN + static_cast<int>(rank) * kGemmBHalf;
-    for (int kb = 0; kb < nkb; ++kb) {
+    for (int kb = kb_begin; kb < kb_end; ++kb) {
       const uint32_t empty_bar = wide ? GemmSmem::wempty(base, wstage) : GemmSmem::empty(base, stage);
       if (!mbar_wait(empty_bar, (wide ? wphase : phase) ^ 1u, abort_flag, p.status)) {
         ok = false;
@@ -249,7 +269,8 @@ __device__ __forceinline__ void gemm_mma(const GemmParams& p, uint32_t base, uin
   for (int j = 0; ok && (u = pair_unit(p, pair, npairs, j)) >= 0; ++j) {
     const UnitCoord uc = decode_unit<kAMode>(p, u);
     const GemmProblem& pr = p.prob[uc.prob];
-    const int nkb = (pr.K + KE - 1) / KE;
+    int kb_begin, kb_end;
+    unit_kblocks<kTF32>(pr, uc, kb_begin, kb_end);
     const bool amn = a_mn_of<kAMode>(pr);
     const bool wide = wide_of<kAMode>(pr);
     const uint32_t idesc = make_idesc(kPairM, kGemmBN, kTF32, amn, kBMN);
@@ -260,7 +281,7 @@ __device__ __forceinline__ void gemm_mma(const GemmParams& p, uint32_t base, uin
     if (!ok) break;
     tc_fence_after();
     const uint32_t d0 = tmem + (tiles & 1u) * kGemmBN, d1 = tmem + ((tiles + 1u) & 1u) * kGemmBN;
-    for (int kb = 0; kb < nkb; ++kb) {
+    for (int kb = kb_begin; kb < kb_end; ++kb) {
       const uint32_t full_bar = wide ? GemmSmem::wfull(base, wstage) : GemmSmem::full(base, stage);
       if (!mbar_wait(full_bar, wide ? wphase : phase, abort_flag, p.status)) {
         ok = false;
@@ -274,13 +295,13 @@ __device__ __forceinline__ void gemm_mma(const GemmParams& p, uint32_t base, uin
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk)
         mma_issue_pair<kTF32>(d0, ad + kk * (amn ? kStepMN : kStepK),
-                              bd + kk * (kBMN ? kStepMN : kStepK), idesc, (kb | kk) != 0);
+                              bd + kk * (kBMN ? kStepMN : kStepK), idesc, kb > kb_begin || kk > 0);
       if (uc.nt == 2) {
         const uint64_t bd1 = operand_desc<kTF32>(sb + kGemmBBytes, kBMN, kBox);  // second column tile
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
           mma_issue_pair<kTF32>(d1, ad + kk * (amn ? kStepMN : kStepK),
-                                bd1 + kk * (kBMN ? kStepMN : kStepK), idesc, (kb | kk) != 0);
+                                bd1 + kk * (kBMN ? kStepMN : kStepK), idesc, kb > kb_begin || kk > 0);
       }
       if (wide) {
         mma_commit_pair(GemmSmem::wempty(base, wstage), kBoth);
@@ -452,7 +473,7 @@ __device__ __forceinline__ void gemm_epilogue(const GemmParams& p, uint32_t base
         epilogue_stats(pr, &p.mapC[uc.prob], stage, stores, tl + acc * kGemmBN, tn, row, row_ok,
                        row0, lane);
       } else {
-        float* crow = pr.C + (row_ok ? row : 0) * pr.ldc;
+        float* crow = pr.C + uc.ks * pr.split_stride + (row_ok ? row : 0) * pr.ldc;
 #pragma unroll 1
         for (int c = 0; c < kGemmBN / 32; ++c) {
           tmem_ld32(tl + acc * kGemmBN + c * 32, v);

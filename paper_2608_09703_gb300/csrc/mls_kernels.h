@@ -140,6 +140,13 @@ struct GemmProblem {
   // and the number of passes over B.  The accumulators are then not double
   // buffered, so this suits problems with a long reduction.
   int wide;
+  // Split reduction (launch_gemm_mixed only, not with wide units): ksplit > 1
+  // units share an output tile, unit `ks` takes the k-blocks [ks kb_split,
+  // (ks + 1) kb_split) and writes its own sum to C + ks * split_stride; the sums
+  // are added afterwards (launch_split_sum).  Units are numbered split by split.
+  int ksplit;                    // 0 or 1: one unit reduces all of K
+  int kb_split;
+  long long split_stride;        // floats between the splits' copies of C
 };
 enum GemmEpilogue { kEpiPlain = 0, kEpiSoftmax = 1, kEpiArgmax = 2 };
 
@@ -319,6 +326,16 @@ cudaError_t launch_gemm_stats(const GemmParams& p, bool tf32, int grid, cudaStre
 cudaError_t launch_merge(const MergeParams& p, int blocks, cudaStream_t s);
 cudaError_t launch_final(const double* block_sum, const long long* block_cnt, int nblocks,
                          float* loss, cudaStream_t s);
+// out_m [rows, cols_m] (+)= sum over s < nsplit of part[s * stride + off_m + ...], for
+// every sub-model, in split order (deterministic); see GemmProblem::ksplit.
+struct SplitSumParams {
+  int nprob, nsplit, accumulate;
+  long long stride;              // floats between splits
+  const float* part[kMaxModels];
+  float* out[kMaxModels];
+  long long n4[kMaxModels];      // float4s of out_m
+};
+cudaError_t launch_split_sum(const SplitSumParams& p, cudaStream_t s);
 cudaError_t launch_count(const int* y, long long T, long long V, float* inv_n, int* status,
                          cudaStream_t s);
 

@@ -271,6 +271,32 @@ __global__ void __launch_bounds__(kFinalThreads)
   if (threadIdx.x == 0) *loss = C > 0.0 ? static_cast<float>(S / C) : 0.f;
 }
 
+// Sums of a split reduction: a thread owns float4s of one sub-model's output
+// (blockIdx.y) and adds the splits' copies in order, so the result does not
+// depend on timing.  Bound by reading the copies (L2, just written).
+constexpr int kSplitSumThreads = 256;
+
+__global__ void __launch_bounds__(kSplitSumThreads)
+    split_sum_kernel(const __grid_constant__ SplitSumParams p) {
+  const int m = blockIdx.y;
+  const long long n4 = p.n4[m], s4 = p.stride / 4;
+  const float4* part = reinterpret_cast<const float4*>(p.part[m]);
+  float4* out = reinterpret_cast<float4*>(p.out[m]);
+  for (long long i = static_cast<long long>(blockIdx.x) * kSplitSumThreads + threadIdx.x; i < n4;
+       i += static_cast<long long>(gridDim.x) * kSplitSumThreads) {
+    float4 a = p.accumulate ? out[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int s = 0; s < p.nsplit; ++s) {
+      const float4 b = part[s * s4 + i];
+      a.x += b.x;
+      a.y += b.y;
+      a.z += b.z;
+      a.w += b.w;
+    }
+    out[i] = a;
+  }
+}
+
 constexpr int kCountThreads = 1024;
 
 __global__ void __launch_bounds__(kCountThreads)
@@ -303,6 +329,16 @@ cudaError_t launch_merge(const MergeParams& p, int blocks, cudaStream_t s) {
 cudaError_t launch_final(const double* block_sum, const long long* block_cnt, int nblocks,
                          float* loss, cudaStream_t s) {
   final_kernel<<<1, kFinalThreads, 0, s>>>(block_sum, block_cnt, nblocks, loss);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_split_sum(const SplitSumParams& p, cudaStream_t s) {
+  long long most = 0;
+  for (int m = 0; m < p.nprob; ++m) most = p.n4[m] > most ? p.n4[m] : most;
+  if (most <= 0) return cudaSuccess;
+  const long long blocks = (most + kSplitSumThreads - 1) / kSplitSumThreads;
+  const dim3 grid(static_cast<unsigned>(blocks < 4096 ? blocks : 4096), p.nprob);
+  split_sum_kernel<<<grid, kSplitSumThreads, 0, s>>>(p);
   return cudaGetLastError();
 }
 

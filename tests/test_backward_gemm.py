@@ -39,3 +39,22 @@ def test_fp32_reads_g_h_w_in_place(T, d, V, vocab_group):
     lie (no K-major copies), in one launch."""
     wl = synth.Workload("fp32", T=T, d=d, V=V, dtype="fp32", tau=0.8, alpha=0.4, w_sigma=0.05)
     grads_match_oracle(wl, seed=21, vocab_group=vocab_group)
+
+
+@pytest.mark.parametrize("dtype,T,d,V,vocab_group", [
+    ("bf16", 70, (64, 136), 20000, 0),      # dH: 2 tiles over 313 k-blocks
+    ("bf16", 70, (64, 136), 20011, 9984),   # three groups: the copies added to dH
+    ("fp32", 33, (36, 100), 9001, 0),
+    ("bf16", 9001, (64, 136), 300, 0),      # dW: 4 tiles over 141 k-blocks of tokens
+    ("fp32", 5000, (36, 100), 257, 0),
+])
+def test_split_reduction(dtype, T, d, V, vocab_group):
+    """A few long reductions, cut into several units each: the last split
+    shorter than the others, and the copies summed into the output."""
+    wl = synth.Workload("split", T=T, d=d, V=V, dtype=dtype, tau=0.8, alpha=0.4, w_sigma=0.05)
+    B.mls_profile_enable(True)
+    try:
+        grads_match_oracle(wl, seed=22, vocab_group=vocab_group)
+        assert "split_sum" in B.mls_profile_read()
+    finally:
+        B.mls_profile_enable(False)
