@@ -417,6 +417,20 @@ int encode(CUtensorMap* map, const void* ptr, int elt, long long cols, long long
   return MLS_OK;
 }
 
+// Row-major fp32 output [copies, rows, cols] of dense rows, `stride` floats
+// between copies, as boxes of 32 x 32 for TMA stores.
+int encode_out(CUtensorMap* map, float* ptr, long long cols, long long rows, int copies,
+               long long stride) {
+  const cuuint64_t dims[3] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows),
+                              static_cast<cuuint64_t>(copies)};
+  const cuuint64_t strides[2] = {static_cast<cuuint64_t>(cols) * 4, static_cast<cuuint64_t>(stride) * 4};
+  const cuuint32_t box[3] = {32, 32, 1}, estr[3] = {1, 1, 1};
+  const CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, ptr, dims, strides, box, estr,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? MLS_OK : fail(MLS_ERR_CUDA, "cuTensorMapEncodeTiled (output)");
+}
+
 void fill_head_common(HeadParams& hp, const mls_problem* p, const Plan& pl, const int* y,
                       int* status) {
   const int KE = 128 / pl.elt;
@@ -656,8 +670,7 @@ extern "C" int mls_head_loss_bwd(const mls_problem* p, const void* const* H, con
       q.K = static_cast<int>(dh ? gc : p->T);
       q.a_map = q.b_map = i;
       q.b_k0 = dh ? static_cast<int>(c0) : 0;
-      q.C = dh ? dH[m] : dW[m] + c0 * p->d[m];
-      q.ldc = p->d[m];
+      float* out = dh ? dH[m] : dW[m] + c0 * p->d[m];
       q.accumulate = dh && g > 0 ? 1 : 0;
       q.a_mn = dh ? 0 : 1;
       q.tiles_m = static_cast<int>(ceil_div(q.Mrows, 2 * kGemmBM));
@@ -668,15 +681,17 @@ extern "C" int mls_head_loss_bwd(const mls_problem* p, const void* const* H, con
       if (is_long && cut.ksplit > 1) {  // the units write their own sums, added up below
         q.ksplit = cut.ksplit;
         q.kb_split = cut.kb_split;
-        q.split_stride = cut.part_floats / cut.ksplit;
-        sum.out[m] = q.C;
+        sum.out[m] = out;
         sum.n4[m] = static_cast<long long>(q.Mrows) * p->d[m] / 4;
         sum.accumulate = q.accumulate;
-        q.C = split_ws + split_off;
+        out = split_ws + split_off;
         q.accumulate = 0;
-        sum.part[m] = q.C;
+        sum.part[m] = out;
         split_off += static_cast<long long>(q.Mrows) * p->d[m];
       }
+      if (encode_out(&gb.mapC[i], out, p->d[m], q.Mrows, q.ksplit > 1 ? q.ksplit : 1,
+                     q.ksplit > 1 ? cut.part_floats / cut.ksplit : static_cast<long long>(q.Mrows) * p->d[m]))
+        return MLS_ERR_CUDA;
       if (i == M - 1) n_long = units;
     }
     gb.nprob = 2 * M;
@@ -1114,8 +1129,6 @@ extern "C" int mls_spec_verify(const mls_spec_problem* p, const void* H_draft, c
     pr.Ncols = static_cast<int>(p->V);
     pr.K = ds[m];
     pr.a_map = pr.b_map = i;
-    pr.C = Cs[m];
-    pr.ldc = pl.ldz;
     pr.tiles_n = static_cast<int>(pl.tiles);
     pr.tiles_m = static_cast<int>(ceil_div(Ps[m], 2 * kGemmBM));
     pr.m_fast = 1;

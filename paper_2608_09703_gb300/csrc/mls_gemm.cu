@@ -59,9 +59,8 @@ struct GemmSmem {
   static constexpr uint32_t kTmemSlot = kBar + 8u * (2 * kGemmStages + 5 + 2 * kGemmWideStages);
   static constexpr uint32_t kAbort = kTmemSlot + 4;
   static constexpr uint32_t kEnd = kAbort + 4;
-  // kEpiSoftmax output staging: per epilogue warp two 32 x 32 fp32 chunks
-  // (128B-swizzled) written out by TMA stores.  It lies in the slack past the
-  // operand stages, which only the MN-major (plain-epilogue) GEMMs over-read.
+  // Output staging: per epilogue warp two 32 x 32 fp32 chunks (128B-swizzled)
+  // written out by TMA stores.  It lies in the slack past the operand stages.
   static constexpr uint32_t kChunk = 32 * 32 * 4;
   static constexpr uint32_t kStaging = (kEnd + 1023u) & ~1023u;
 };
@@ -465,41 +464,42 @@ __device__ __forceinline__ void gemm_epilogue(const GemmParams& p, uint32_t base
         break;
       }
       tc_fence_after();
-      const long long row = static_cast<long long>(uc.tm) * kPairM + rank * kGemmBM + warp * 32 + lane;
-      const bool row_ok = row < pr.Mrows;
       float v[32];
       if (kStats && pr.epi != kEpiPlain) {
         const int row0 = uc.tm * kPairM + static_cast<int>(rank) * kGemmBM + warp * 32;
-        epilogue_stats(pr, &p.mapC[uc.prob], stage, stores, tl + acc * kGemmBN, tn, row, row_ok,
-                       row0, lane);
+        const long long row = static_cast<long long>(row0) + lane;
+        epilogue_stats(pr, &p.mapC[uc.prob], stage, stores, tl + acc * kGemmBN, tn, row,
+                       row < pr.Mrows, row0, lane);
       } else {
-        float* crow = pr.C + uc.ks * pr.split_stride + (row_ok ? row : 0) * pr.ldc;
+        // 32 x 32 chunks through two staging buffers of this warp, written by TMA
+        // stores (which drop what lies outside C), so that whole 128-byte lines
+        // leave the SM.  One row per thread with 16-byte stores took about 13 us
+        // per 256x256 tile, more than the MMAs of a tile with K < 2500.
+        const int row0 = uc.tm * kPairM + static_cast<int>(rank) * kGemmBM + warp * 32;
+        const int ncols = row0 < pr.Mrows ? pr.Ncols - tn * kGemmBN : 0;
 #pragma unroll 1
-        for (int c = 0; c < kGemmBN / 32; ++c) {
+        for (int c = 0; c * 32 < kGemmBN && c * 32 < ncols; ++c) {
           tmem_ld32(tl + acc * kGemmBN + c * 32, v);
-          const int col = tn * kGemmBN + c * 32;
-          if (row_ok && col < pr.Ncols) {
-            float* dst = crow + col;
-            if (col + 32 <= pr.Ncols) {
-              float4* d4 = reinterpret_cast<float4*>(dst);
+          const uint32_t buf = stage + (stores & 1u) * GemmSmem::kChunk;
+          if (lane == 0) bulk_wait_read<1>();  // the store that last used this buffer has read it
+          __syncwarp();
+          const uint32_t rowaddr = buf + lane * 128;
 #pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                float4 o = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-                if (pr.accumulate) {
-                  const float4 c4 = d4[i];
-                  o.x += c4.x;
-                  o.y += c4.y;
-                  o.z += c4.z;
-                  o.w += c4.w;
-                }
-                d4[i] = o;
-              }
-            } else {
-#pragma unroll
-              for (int i = 0; i < 32; ++i)
-                if (col + i < pr.Ncols) dst[i] = pr.accumulate ? dst[i] + v[i] : v[i];
-            }
+          for (int q = 0; q < 8; ++q)
+            st_shared_v4(rowaddr + ((q ^ (lane & 7)) << 4), __float_as_uint(v[4 * q]),
+                         __float_as_uint(v[4 * q + 1]), __float_as_uint(v[4 * q + 2]),
+                         __float_as_uint(v[4 * q + 3]));
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            const int col = tn * kGemmBN + c * 32;
+            if (pr.accumulate)
+              tma_reduce_add_3d(&p.mapC[uc.prob], buf, col, row0, uc.ks);
+            else
+              tma_store_3d(&p.mapC[uc.prob], buf, col, row0, uc.ks);
+            bulk_commit();
           }
+          ++stores;
         }
       }
       tc_fence_before();

@@ -115,9 +115,7 @@ struct GemmProblem {
   int Mrows, Ncols, K;           // C is Mrows x Ncols, reduction length K
   int a_map, b_map;              // index into mapA / mapB
   int a_m0, a_k0, b_n0, b_k0;    // coordinate offsets into the tensors
-  float* C;                      // row-major fp32, leading dimension ldc
-  long long ldc;
-  int accumulate;                // C += A*B if 1, C = A*B if 0
+  int accumulate;                // C += A*B if 1, C = A*B if 0 (C is mapC)
   int tiles_n;                   // ceil(Ncols / kGemmBN)
   int tile_begin;                // first unit of this problem in the launch's unit numbering
                                  // (a unit is one pair tile of 256 x kGemmBN, or two if wide)
@@ -142,11 +140,10 @@ struct GemmProblem {
   int wide;
   // Split reduction (launch_gemm_mixed only, not with wide units): ksplit > 1
   // units share an output tile, unit `ks` takes the k-blocks [ks kb_split,
-  // (ks + 1) kb_split) and writes its own sum to C + ks * split_stride; the sums
-  // are added afterwards (launch_split_sum).  Units are numbered split by split.
+  // (ks + 1) kb_split) and writes its own sum to copy ks of C; the copies are
+  // added afterwards (launch_split_sum).  Units are numbered split by split.
   int ksplit;                    // 0 or 1: one unit reduces all of K
   int kb_split;
-  long long split_stride;        // floats between the splits' copies of C
 };
 enum GemmEpilogue { kEpiPlain = 0, kEpiSoftmax = 1, kEpiArgmax = 2 };
 
@@ -155,7 +152,9 @@ constexpr int kGemmMaxProblems = 2 * kMaxModels;
 struct GemmParams {
   CUtensorMap mapA[kGemmMaxProblems];
   CUtensorMap mapB[kGemmMaxProblems];
-  CUtensorMap mapC[kGemmMaxProblems];  // kEpiSoftmax: C fp32 [Mrows, Ncols], box {32, 32}, 128B swizzle
+  // C fp32, 128B swizzle.  kEpiPlain: [ksplit, Mrows, Ncols], box {32, 32, 1};
+  // kEpiSoftmax: [Mrows, Ncols], box {32, 32}.
+  CUtensorMap mapC[kGemmMaxProblems];
   int nprob;
   GemmProblem prob[kGemmMaxProblems];
   int total_tiles;               // units of the launch (pair tiles, or pairs of them if wide)
