@@ -25,7 +25,7 @@ LIB = os.path.join(PKG, "libmls.so")
 BUILD_CHECKED = os.path.join(PKG, "_build_checked")
 LIB_CHECKED = os.path.join(PKG, "libmls_checked.so")
 SOURCES = ["mls_api.cu", "mls_head.cu", "mls_gemm.cu", "mls_reduce.cu", "mls_eval.cu",
-           "mls_junction.cu", "mls_spec.cu"]
+           "mls_junction.cu", "mls_spec.cu", "mls_logits.cu"]
 HEADERS = ["mls_device.cuh", "mls_kernels.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -70,6 +70,8 @@ int device_state(DeviceState** out) {
       s.err = fail(MLS_ERR_CUDA, "eval kernel attributes", e);
     } else if ((e = setup_spec_kernels()) != cudaSuccess) {
       s.err = fail(MLS_ERR_CUDA, "spec kernel attributes", e);
+    } else if ((e = setup_logits_kernels()) != cudaSuccess) {
+      s.err = fail(MLS_ERR_CUDA, "logits kernel attributes", e);
     } else if ((e = setup_junction_kernels()) != cudaSuccess) {
       s.err = fail(MLS_ERR_CUDA, "junction kernel attributes", e);
     } else if ((s.gemm_pairs = gemm_max_active_pairs()) <= 0) {
@@ -1004,6 +1006,7 @@ extern "C" int mls_junction_bwd(int64_t T, int32_t d_prev, int32_t d_next, int32
 namespace {
 struct SpecPlan {
   long long Pd = 0, Pv = 0, ldz = 0, tiles = 0;
+  bool few = false;     // few rows: logits by mls_logits.cu, tiles of kLogitsTile columns
   size_t off_ev = 0, off_ed = 0, off_sv = 0, off_sd = 0, off_fv = 0, off_fd = 0;
   size_t off_stv = 0, off_std = 0, total = 0;
 };
@@ -1031,7 +1034,11 @@ SpecPlan spec_plan(const mls_spec_problem* p) {
   pl.Pv = static_cast<long long>(p->B) * (p->gamma + 1);
   pl.Pd = p->greedy ? 0 : static_cast<long long>(p->B) * p->gamma;
   pl.ldz = ceil_div(p->V, 4) * 4;
-  pl.tiles = ceil_div(p->V, kGemmBN);
+  // Few rows: bound by reading the heads (mls_logits.cu says more; at its
+  // largest, 128 rows, the launch takes 83 us against the pair GEMM's 92).
+  // Sampling keeps a row's tile table in shared memory, hence the bound on V.
+  pl.few = pl.Pv <= kLogitsMaxRows && p->V <= static_cast<long long>(kSpecMaxTiles) * kLogitsTile;
+  pl.tiles = ceil_div(p->V, pl.few ? kLogitsTile : kGemmBN);
   const size_t rows_e = p->greedy ? 0 : static_cast<size_t>(pl.Pv);  // e_t is only stored when sampling
   size_t o = 0;
   auto take = [&](size_t& off, size_t bytes) {
@@ -1088,6 +1095,7 @@ extern "C" int mls_spec_verify(const mls_spec_problem* p, const void* H_draft, c
   sp.gamma = p->gamma;
   sp.greedy = p->greedy ? 1 : 0;
   sp.tiles = static_cast<int>(pl.tiles);
+  sp.tile_shift = pl.few ? 7 : 8;
   sp.scale = p->greedy ? 1.f : 1.4426950408889634f / p->temperature;
   sp.top_p = p->greedy ? 1.f : p->top_p;
   sp.ev = at(pl.off_ev);
@@ -1103,19 +1111,53 @@ extern "C" int mls_spec_verify(const mls_spec_problem* p, const void* H_draft, c
   sp.n_accepted = n_accepted;
   sp.next_token = next_token;
   sp.status = dev->status;
+  sp.sms = dev->sms;
 
-  // Logits of the verify positions: one GEMM launch over the verifier's rows
-  // and (sampling) the draft's, z = H W^T with both operands K-major; its
-  // epilogue leaves per-tile softmax statistics (sampling) or the per-tile
-  // maximum and argmax (greedy) instead of the logits.
-  GemmParams g;
-  std::memset(&g, 0, sizeof g);
+  // Logits of the verify positions: one launch over the verifier's rows and
+  // (sampling) the draft's, z = H W^T with both operands K-major; its epilogue
+  // leaves per-tile softmax statistics (sampling) or the per-tile maximum and
+  // argmax (greedy) instead of the logits.
   const void* Hs[2] = {H_verify, H_draft};
   const void* Ws[2] = {W_verify, W_draft};
   const int ds[2] = {p->d_verify, p->d_draft};
   const long long Ps[2] = {pl.Pv, pl.Pd};
   float* Cs[2] = {at(pl.off_ev), at(pl.off_ed)};
   float* Ss[2] = {at(pl.off_stv), at(pl.off_std)};
+  if (pl.few) {
+    LogitsParams lp;
+    std::memset(&lp, 0, sizeof lp);
+    const int first = Ps[1] > 0 && ds[1] > ds[0] ? 1 : 0;
+    lp.n = static_cast<int>(ceil_div(pl.Pv, 16) * 16);
+    for (int k = 0; k < 2; ++k) {
+      const int m = k == 0 ? first : 1 - first;
+      if (Ps[m] == 0) continue;
+      const int i = lp.nprob++;
+      if (encode(&lp.mapW[i], Ws[m], elt, ds[m], p->V, ds[m], KE, kLogitsTile) ||
+          encode(&lp.mapH[i], Hs[m], elt, ds[m], Ps[m], ds[m], KE, lp.n))
+        return MLS_ERR_CUDA;
+      lp.prob[i] = {static_cast<int>(Ps[m]), static_cast<int>(ceil_div(ds[m], KE)),
+                    static_cast<int>(pl.tiles), Cs[m], Ss[m]};
+    }
+    lp.greedy = sp.greedy;
+    lp.scale = sp.scale;
+    lp.V = p->V;
+    lp.ldz = pl.ldz;
+    lp.stats_ld = 2 * pl.tiles;
+    lp.status = dev->status;
+    const int units = static_cast<int>(pl.tiles) * lp.nprob;
+    const int grid = units < dev->sms ? units : dev->sms;
+    const int r = lp.prob[0].tiles % grid;
+    if (lp.nprob > 1 && r > 0) {
+      const long long fair = ceil_div(lp.prob[1].tiles, grid - r);
+      const long long even = ceil_div(lp.prob[0].nk, lp.prob[1].nk);
+      lp.catchup = static_cast<int>(fair < even ? fair : even);
+    }
+    if ((rc = timed("spec_logits", s, [&] { return launch_logits(lp, tf32, grid, s); }))) return rc;
+    if (!p->greedy && (rc = timed("spec_rows", s, [&] { return launch_spec_rows(sp, s); }))) return rc;
+    return timed("spec_sample", s, [&] { return launch_spec_sample(sp, s); });
+  }
+  GemmParams g;
+  std::memset(&g, 0, sizeof g);
   int tiles = 0;
   for (int m = 0; m < 2; ++m) {
     if (Ps[m] == 0) continue;

@@ -265,7 +265,8 @@ struct SpecParams {
   long long V, ldz;
   int B, gamma;
   int greedy;
-  int tiles;                     // column tiles of kGemmBN per row
+  int tiles;                     // column tiles of 2^tile_shift per row
+  int tile_shift;                // 8 (the pair GEMM's kGemmBN) or 7 (kLogitsTile)
   float scale;                   // log2(e) / temperature
   float top_p;
   const float* ed;               // [B * gamma][ldz] draft e_t (sampling only)
@@ -281,7 +282,31 @@ struct SpecParams {
   int* n_accepted;               // [B]
   int* next_token;               // [B]
   int* status;                   // checked build: invariant failures
+  int sms;                       // SMs of the device
 };
+// Logits of few rows (mls_logits.cu): both sub-models' rows against their whole
+// heads in one launch, with the outputs of the GEMM's statistics epilogues.
+constexpr int kLogitsMaxRows = 128;
+constexpr int kLogitsTile = 128;       // vocabulary columns of a unit and of its statistics
+struct LogitsProblem {
+  int rows, nk, tiles;           // rows of H, k-blocks of 128 bytes, column tiles
+  float* e;                      // [rows][ldz] e_t (sampling only)
+  float* stats;                  // [rows][stats_ld]: per tile (m_t, sum) or (m_t, argmax)
+};
+struct LogitsParams {
+  CUtensorMap mapW[2];           // W [V, d], box {128 B of K, kLogitsTile rows}
+  CUtensorMap mapH[2];           // H [rows, d], box {128 B of K, n rows}
+  int nprob;                     // 1 or 2, the longer reduction first
+  LogitsProblem prob[2];
+  int n;                         // MMA columns: the larger row count rounded up to 16
+  int catchup;                   // second-problem units that CTAs one first-problem unit short take
+  int greedy;
+  float scale;                   // log2(e) / temperature
+  long long V, ldz, stats_ld;
+  int* status;
+};
+cudaError_t setup_logits_kernels();
+cudaError_t launch_logits(const LogitsParams& p, bool tf32, int grid, cudaStream_t s);
 cudaError_t setup_spec_kernels();
 cudaError_t launch_spec_rows(const SpecParams& p, cudaStream_t s);
 cudaError_t launch_spec_sample(const SpecParams& p, cudaStream_t s);

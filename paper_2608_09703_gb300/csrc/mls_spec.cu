@@ -11,8 +11,8 @@
 // cumulative probability reaches top_p, then renormalised.  Greedy: accept
 // while x_i == argmax of the verifier's logits (lowest index on ties).
 //
-// The logits GEMM's epilogue (mls_gemm.cu) leaves, per row and column tile t
-// of 256, e_t[v] = 2^((z[v] - m_t) log2(e) / T) and (m_t, sum_t), or for greedy
+// The logits launch (mls_gemm.cu, or mls_logits.cu for few rows) leaves, per
+// row and column tile t of 256 (128) = 2^tsh, e_t[v] = 2^((z[v] - m_t) log2(e) / T) and (m_t, sum_t), or for greedy
 // only (m_t, argmax_t).  Here, with m = max_t m_t and f_t = 2^((m_t - m) log2(e)/T),
 // every token's unnormalised probability is e[v] = e_t[v] f_t (<= 1) and
 // S = sum_t sum_t f_t:
@@ -35,15 +35,13 @@
 namespace mls {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
-constexpr int kStep = 128;              // elements one warp covers per float4 step
+constexpr int kStepShift = 7;
+constexpr int kStep = 1 << kStepShift;  // elements one warp covers per float4 step
 constexpr int kUnroll = 6;              // independent float4 loads in flight per lane
 constexpr int kFinish = 256;            // candidates resolved exactly
 constexpr uint32_t kOneKey = 0x3f800000u;     // bit pattern of 1.0f
 constexpr uint32_t kFirstMid = 0x3b800000u;   // 2^-8
 constexpr uint32_t kSecondMid = 0x37800000u;  // 2^-16
-static_assert(kFinish <= kThreads, "one candidate per thread in the exact finish");
 
 // Per-warp partials of a block reduction (f, n, k) and the combined results
 // (rf, rn, rk) that warp 0 writes for everyone.
@@ -58,7 +56,6 @@ struct SharedT {
   int rn[3];
   uint32_t rk[4];
 };
-using Shared = SharedT<kWarps>;
 constexpr int kSampleWarps = 32;  // the per-sequence sampler runs 1024 threads
 
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
@@ -179,15 +176,16 @@ __device__ uint32_t block_max_u(uint32_t v, SharedT<NW>& sh) {
 
 // Per-row softmax statistics from the per-tile ones: m, S and f_t (into the
 // shared table and, if fg is not null, into global memory).
+template <int NW>
 __device__ void row_stats(const float* st, int tiles, float scale, float* ftab, float* fg,
-                          float& m, float& S, Shared& sh) {
+                          float& m, float& S, SharedT<NW>& sh) {
   float mv = -INFINITY;
   int unused = 0;
-  for (int t = threadIdx.x; t < tiles; t += kThreads) mv = fmaxf(mv, st[2 * t]);
+  for (int t = threadIdx.x; t < tiles; t += NW * 32) mv = fmaxf(mv, st[2 * t]);
   block_argmax(mv, unused, sh);
   m = mv;
   float s = 0.f;
-  for (int t = threadIdx.x; t < tiles; t += kThreads) {
+  for (int t = threadIdx.x; t < tiles; t += NW * 32) {
     const float f = fast_exp2((st[2 * t] - m) * scale);
     ftab[t] = f;
     if (fg) fg[t] = f;
@@ -203,7 +201,7 @@ __device__ void row_stats(const float* st, int tiles, float scale, float* ftab, 
 // at or past V are not meaningful).  The loop is warp-uniform, so f may use
 // warp collectives.  Rows are 16-byte aligned and padded to 4 elements.
 template <int NW, typename F>
-__device__ __forceinline__ void for_row(const float* et, const float* ftab, long long V, F&& f) {
+__device__ __forceinline__ void for_row(const float* et, const float* ftab, int tsh, long long V, F&& f) {
   const int l = lane_id();
   constexpr long long kStride = static_cast<long long>(NW) * kStep;
   for (long long base = static_cast<long long>(warp_id()) * kStep; base < V;
@@ -219,7 +217,7 @@ __device__ __forceinline__ void for_row(const float* et, const float* ftab, long
     for (int u = 0; u < kUnroll; ++u) {
       const long long i0 = base + u * kStride + l * 4;
       if (i0 < V) {
-        const float fm = ftab[i0 / kGemmBN];
+        const float fm = ftab[i0 >> tsh];
         v[u].x *= fm;
         v[u].y *= fm;
         v[u].z *= fm;
@@ -263,18 +261,18 @@ struct PassStats {
 // One bisection pass over a whole row (e = e_t f_t), warps taking 128-token
 // steps w, w + 16, ..., kUnroll steps per iteration; only the row's last
 // float4 can be partial.
-template <bool kTrack>
-__device__ __forceinline__ void row_pass(const float* et, const float* ftab, int V, uint32_t lo,
+template <bool kTrack, int NW>
+__device__ __forceinline__ void row_pass(const float* et, const float* ftab, int tsh, int V, uint32_t lo,
                                          uint32_t mo, uint32_t wm, PassStats& ps) {
   const int l = lane_id();
-  constexpr int kStride = kWarps * kStep;
+  constexpr int kStride = NW * kStep;
   for (int base = warp_id() * kStep; base < V; base += kUnroll * kStride) {
     float4 v[kUnroll];
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
       const int s0 = base + u * kStride, i0 = s0 + l * 4;
       // a tile whose maximum lies below the bracket holds no candidate
-      const bool live = s0 < V && __float_as_uint(ftab[static_cast<unsigned>(s0) / kGemmBN]) >= lo;
+      const bool live = s0 < V && __float_as_uint(ftab[s0 >> tsh]) >= lo;
       v[u] = live && i0 < V ? __ldg(reinterpret_cast<const float4*>(et + i0))
                             : make_float4(0.f, 0.f, 0.f, 0.f);
     }
@@ -282,7 +280,7 @@ __device__ __forceinline__ void row_pass(const float* et, const float* ftab, int
     for (int u = 0; u < kUnroll; ++u) {
       const int i0 = base + u * kStride + l * 4;
       if (i0 < V) {
-        const float fm = ftab[static_cast<unsigned>(i0) / kGemmBN];
+        const float fm = ftab[i0 >> tsh];
         if (__float_as_uint(fm) < lo) continue;
         const float e0 = v[u].x * fm, e1 = v[u].y * fm, e2 = v[u].z * fm, e3 = v[u].w * fm;
         ps.add<kTrack>(e0, lo, mo, wm);
@@ -327,73 +325,67 @@ __device__ int kept_tiles(const float* ftab, int tiles, uint32_t min_key, int* k
 }
 
 // The first bisection pass over a row: the split at 2^-8 of the maximum.
-// Only the kept tiles are read.  Warp w takes kept[w], kept[w + kWarps], ...,
-// kFirstTiles of them per round with all their loads in flight, so a peaked
-// row (a few dozen kept tiles spread over the vocabulary) costs about one
-// memory latency.  Mass and count of the upper side; its few tokens are also
+// Only the kept tiles are read, kFirstSteps steps of 128 per warp and round with
+// all their loads in flight, so a peaked row (a few dozen kept tiles spread over
+// the vocabulary) costs about one memory latency.  Mass and count of the upper side; its few tokens are also
 // appended, in this warp's visiting order, to its own region of
-// kSpecListCap / kWarps slots of `regions` (wrun counts them, also past the
+// kSpecListCap / NW slots of `regions` (wrun counts them, also past the
 // region's end).
-constexpr int kRegion = kSpecListCap / kWarps;
-constexpr int kFirstTiles = 3;
-static_assert(kGemmBN == 2 * kStep, "a column tile is two 128-element steps");
-__device__ __forceinline__ void first_pass(const float* et, const float* ftab, const int* kept,
+constexpr int kFirstSteps = 6;  // in flight per warp and round
+template <int NW>
+__device__ __forceinline__ void first_pass(const float* et, const float* ftab, int tsh, const int* kept,
                                            int nk, int V, float* regions, PassStats& ps,
                                            int& wrun) {
-  const int l = lane_id();
+  constexpr int kRegion = kSpecListCap / NW;
+  const int l = lane_id(), sub = tsh - kStepShift;
+  const int ns = nk << sub;  // steps of the kept tiles
   float* reg = regions + warp_id() * kRegion;
   wrun = 0;
-  for (int j0 = warp_id(); j0 < nk; j0 += kFirstTiles * kWarps) {
-    float4 v[kFirstTiles][2];
-    float fm[kFirstTiles];
-    int i0s[kFirstTiles];
+  // Step q of a round: pairs of steps, so that a warp takes whole 256-column tiles.
+  auto step = [&](int q0, int u) { return q0 + (u >> 1) * 2 * NW + (u & 1); };
+  for (int q0 = 2 * warp_id(); q0 < ns; q0 += kFirstSteps * NW) {
+    float4 v[kFirstSteps];
+    float fm[kFirstSteps];
+    int i0s[kFirstSteps];
 #pragma unroll
-    for (int u = 0; u < kFirstTiles; ++u) {
-      const int j = j0 + u * kWarps;
+    for (int u = 0; u < kFirstSteps; ++u) {
+      const int q = step(q0, u);
       fm[u] = 0.f;
       i0s[u] = V;
-      v[u][0] = v[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (j < nk) {  // warp-uniform
-        const int t = kept[j];
+      v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (q < ns) {  // warp-uniform
+        const int t = kept[q >> sub];
         fm[u] = ftab[t];
-        i0s[u] = t * kGemmBN + l * 4;
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-          if (i0s[u] + h * kStep < V)
-            v[u][h] = __ldg(reinterpret_cast<const float4*>(et + i0s[u] + h * kStep));
+        i0s[u] = (t << tsh) + (q & ((1 << sub) - 1)) * kStep + l * 4;
+        if (i0s[u] < V) v[u] = __ldg(reinterpret_cast<const float4*>(et + i0s[u]));
       }
     }
 #pragma unroll
-    for (int u = 0; u < kFirstTiles; ++u) {
-      if (j0 + u * kWarps >= nk) break;  // warp-uniform
+    for (int u = 0; u < kFirstSteps; ++u) {
+      if (step(q0, u) >= ns) break;  // warp-uniform
+      const int nv = min(max(V - i0s[u], 0), 4);
+      const float e[4] = {v[u].x * fm[u], v[u].y * fm[u], v[u].z * fm[u], v[u].w * fm[u]};
+      bool ge[4];
+      int k = 0;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int i0 = i0s[u] + h * kStep;
-        const int nv = min(max(V - i0, 0), 4);
-        const float e[4] = {v[u][h].x * fm[u], v[u][h].y * fm[u], v[u][h].z * fm[u],
-                            v[u][h].w * fm[u]};
-        bool ge[4];
-        int k = 0;
+      for (int j = 0; j < 4; ++j) {
+        ge[j] = j < nv && __float_as_uint(e[j]) >= kFirstMid;
+        if (ge[j]) {
+          ps.mass_ge += e[j];
+          ++k;
+        }
+      }
+      ps.cnt_ge += k;
+      if (__any_sync(0xffffffffu, k > 0)) {
+        const int incl = warp_incl_scan(k);
+        int at = wrun + incl - k;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          ge[j] = j < nv && __float_as_uint(e[j]) >= kFirstMid;
+        for (int j = 0; j < 4; ++j)
           if (ge[j]) {
-            ps.mass_ge += e[j];
-            ++k;
+            if (at < kRegion) reg[at] = e[j];
+            ++at;
           }
-        }
-        ps.cnt_ge += k;
-        if (__any_sync(0xffffffffu, k > 0)) {
-          const int incl = warp_incl_scan(k);
-          int at = wrun + incl - k;
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (ge[j]) {
-              if (at < kRegion) reg[at] = e[j];
-              ++at;
-            }
-          wrun += __shfl_sync(0xffffffffu, incl, 31);
-        }
+        wrun += __shfl_sync(0xffffffffu, incl, 31);
       }
     }
   }
@@ -401,17 +393,18 @@ __device__ __forceinline__ void first_pass(const float* et, const float* ftab, c
 
 // Writes the row's tokens with key in [lo, lo + w) to dst in warp order,
 // this warp from slot `run`, never past cnt.
-__device__ __forceinline__ void row_compact(const float* et, const float* ftab, int V, uint32_t lo,
+template <int NW>
+__device__ __forceinline__ void row_compact(const float* et, const float* ftab, int tsh, int V, uint32_t lo,
                                             uint32_t w, float* dst, int run, int cnt, int* status) {
   const int l = lane_id();
-  constexpr int kStride = kWarps * kStep;
+  constexpr int kStride = NW * kStep;
   for (int base = warp_id() * kStep; base < V; base += kUnroll * kStride) {
     float4 v[kUnroll];
     float fm[kUnroll];
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
       const int s0 = base + u * kStride, i0 = s0 + l * 4;
-      fm[u] = s0 < V ? ftab[static_cast<unsigned>(s0) / kGemmBN] : 0.f;  // warp-uniform
+      fm[u] = s0 < V ? ftab[s0 >> tsh] : 0.f;  // warp-uniform
       v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (__float_as_uint(fm[u]) >= lo && i0 < V) v[u] = __ldg(reinterpret_cast<const float4*>(et + i0));
     }
@@ -442,7 +435,8 @@ __device__ __forceinline__ void row_compact(const float* et, const float* ftab, 
 
 // Block-wide combination; the per-warp counts stay in sh.n[w][1] (upper) and
 // sh.n[w][2] (lower) for the compaction that may follow.
-__device__ void reduce_pass(PassStats& s, Shared& sh) {
+template <int NW>
+__device__ void reduce_pass(PassStats& s, SharedT<NW>& sh) {
   const unsigned full = 0xffffffffu;
   s.mass_ge = warp_sum(s.mass_ge);
   s.cnt_ge = static_cast<int>(__reduce_add_sync(full, static_cast<unsigned>(s.cnt_ge)));
@@ -465,10 +459,10 @@ __device__ void reduce_pass(PassStats& s, Shared& sh) {
   __syncthreads();
   if (warp_id() == 0) {
     const int l = lane_id();
-    const bool has = l < kWarps;
+    const bool has = l < NW;
     float m = has ? sh.f[l][0] : 0.f;
 #pragma unroll
-    for (int o = kWarps / 2; o > 0; o >>= 1) m += __shfl_xor_sync(full, m, o);
+    for (int o = NW / 2; o > 0; o >>= 1) m += __shfl_xor_sync(full, m, o);
     const unsigned cg = __reduce_add_sync(full, has ? static_cast<unsigned>(sh.n[l][1]) : 0u);
     const unsigned cl = __reduce_add_sync(full, has ? static_cast<unsigned>(sh.n[l][2]) : 0u);
     const uint32_t a = __reduce_min_sync(full, has ? sh.k[l][0] : 0xffffffffu);
@@ -497,10 +491,11 @@ __device__ void reduce_pass(PassStats& s, Shared& sh) {
 
 // After reduce_pass: each warp's first output slot when the survivors of
 // side `side` (1 = upper, 2 = lower) are compacted in warp order.
-__device__ __forceinline__ void warp_bases(int side, Shared& sh) {
+template <int NW>
+__device__ __forceinline__ void warp_bases(int side, SharedT<NW>& sh) {
   if (threadIdx.x == 0) {
     int acc = 0;
-    for (int w = 0; w < kWarps; ++w) {
+    for (int w = 0; w < NW; ++w) {
       sh.wbase[w] = acc;
       acc += sh.n[w][side];
     }
@@ -518,8 +513,9 @@ struct RowNucleus {
 // mass(e >= key) = mass_hi + sum of the candidates >= it reaches the target
 // (each candidate's sum is taken over L in index order, so it is monotone in
 // the key), then the mass above b and the ties at b.
+template <int NW>
 __device__ void finish_exact(const float* L, int n, float target, float mass_hi, uint32_t lo,
-                             uint32_t& b, float& gt, int& eq, Shared& sh) {
+                             uint32_t& b, float& gt, int& eq, SharedT<NW>& sh) {
   const int t = threadIdx.x;
   uint32_t kt = 0, best = 0;
   float et = 0.f;
@@ -543,9 +539,11 @@ __device__ void finish_exact(const float* L, int n, float target, float mass_hi,
 }
 
 // Nucleus of one row (e_t, per-tile stats st); writes f_t to fg.
-__device__ RowNucleus nucleus(const float* et, const float* st, float* fg, long long V, int tiles,
+template <int NW>
+__device__ RowNucleus nucleus(const float* et, const float* st, float* fg, long long V, int tiles, int tsh,
                               float scale, float top_p, float* ftab, float* listA, float* listB,
-                              Shared& sh, int* status) {
+                              SharedT<NW>& sh, int* status) {
+  constexpr int kRegion = kSpecListCap / NW;
   RowNucleus r;
   row_stats(st, tiles, scale, ftab, fg, r.m, r.S, sh);
   const float target = top_p * r.S;
@@ -566,7 +564,7 @@ __device__ RowNucleus nucleus(const float* et, const float* st, float* fg, long 
       // The kept-tile list lives in listB until the upper side is copied there.
       int* kept = reinterpret_cast<int*>(listB);
       const int nk = kept_tiles(ftab, tiles, kFirstMid, kept, sh);
-      first_pass(et, ftab, kept, nk, static_cast<int>(V), listA, ps, wrun);
+      first_pass<NW>(et, ftab, tsh, kept, nk, static_cast<int>(V), listA, ps, wrun);
       if (lane_id() == 0) sh.wcnt[warp_id()] = wrun;
       reduce_pass(ps, sh);  // its barriers also publish wcnt
       int cnt;
@@ -575,7 +573,7 @@ __device__ RowNucleus nucleus(const float* et, const float* st, float* fg, long 
         lo = kFirstMid;
         // the upper side is in the warps' regions unless one overflowed
         bool fits = true;
-        for (int w = 0; w < kWarps; ++w) fits = fits && sh.wcnt[w] <= kRegion;
+        for (int w = 0; w < NW; ++w) fits = fits && sh.wcnt[w] <= kRegion;
         if (fits) {
           int at = 0;
           for (int w = 0; w < warp_id(); ++w) at += sh.wcnt[w];
@@ -613,9 +611,9 @@ __device__ RowNucleus nucleus(const float* et, const float* st, float* fg, long 
       const uint32_t mo = mid - lo, wm = hi - mid;
       PassStats ps;
       if (list != nullptr) {
-        for (int i = threadIdx.x; i < n_list; i += kThreads) ps.add<true>(list[i], lo, mo, wm);
+        for (int i = threadIdx.x; i < n_list; i += NW * 32) ps.add<true>(list[i], lo, mo, wm);
       } else {
-        row_pass<false>(et, ftab, static_cast<int>(V), lo, mo, wm, ps);
+        row_pass<false, NW>(et, ftab, tsh, static_cast<int>(V), lo, mo, wm, ps);
       }
       reduce_pass(ps, sh);
       int side, cnt;
@@ -658,9 +656,9 @@ __device__ RowNucleus nucleus(const float* et, const float* st, float* fg, long 
         warp_bases(side, sh);
         int run = sh.wbase[warp_id()];
         if (list == nullptr) {
-          row_compact(et, ftab, static_cast<int>(V), lo, hi - lo, dst, run, cnt, status);
+          row_compact<NW>(et, ftab, tsh, static_cast<int>(V), lo, hi - lo, dst, run, cnt, status);
         } else {
-          for (int base = warp_id() * 32; base < n_list; base += kThreads) {
+          for (int base = warp_id() * 32; base < n_list; base += NW * 32) {
             const int i = base + lane_id();
             float e = 0.f;
             bool keep = false;
@@ -691,7 +689,7 @@ __device__ RowNucleus nucleus(const float* et, const float* st, float* fg, long 
   if (!resolved) {  // top_p = 1, or the rounding exit: one more pass over the row
     float g = 0.f;
     int q = 0;
-    for_row<kWarps>(et, ftab, V, [&](long long i0, const float4& v, long long n) {
+    for_row<NW>(et, ftab, tsh, V, [&](long long i0, const float4& v, long long n) {
 #pragma unroll
       for (int j = 0; j < 4; ++j)
         if (i0 + j < n) {
@@ -718,9 +716,9 @@ __device__ RowNucleus nucleus(const float* et, const float* st, float* fg, long 
 // Nucleus probability of token x (block-wide: when x is tied at the boundary
 // and only some ties are kept, its rank among them is counted).
 template <int NW>
-__device__ float prob_of(const float* et, const float* ftab, long long V, const RowNucleus& n,
+__device__ float prob_of(const float* et, const float* ftab, int tsh, long long V, const RowNucleus& n,
                          int x, SharedT<NW>& sh) {
-  const float e = et[x] * ftab[x / kGemmBN];
+  const float e = et[x] * ftab[x >> tsh];
   bool member = e > n.b;
   if (e == n.b) {
     if (n.c >= n.eq) {
@@ -728,7 +726,7 @@ __device__ float prob_of(const float* et, const float* ftab, long long V, const 
     } else {
       float unused = 0.f;
       int below = 0;
-      for_row<NW>(et, ftab, V, [&](long long i0, const float4& v, long long cnt) {
+      for_row<NW>(et, ftab, tsh, V, [&](long long i0, const float4& v, long long cnt) {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
           if (i0 + j < x && i0 + j < cnt && comp(v, j) == n.b) ++below;
@@ -767,9 +765,11 @@ __host__ __device__ __forceinline__ size_t row_smem(int tiles) {
 
 // One CTA per logits row: rows [0, B (gamma + 1)) are the verifier's, the
 // rest the draft's.  Leaves the row's nucleus state and its f_t table.
-__global__ void __launch_bounds__(kThreads, 4) spec_row_kernel(const SpecParams p) {
+template <int NW>
+__global__ void __launch_bounds__(NW * 32, 32 / NW) spec_row_kernel(const SpecParams p) {
+  static_assert(kFinish <= NW * 32, "one candidate per thread in the exact finish");
   extern __shared__ __align__(16) float smem[];
-  __shared__ Shared sh;
+  __shared__ SharedT<NW> sh;
   const int tiles_pad = (p.tiles + 3) / 4 * 4;
   float* ftab = smem;
   float* listA = smem + tiles_pad;
@@ -780,8 +780,8 @@ __global__ void __launch_bounds__(kThreads, 4) spec_row_kernel(const SpecParams 
   const bool verifier = r < Pv;
   if (!verifier) r -= Pv;
   const float* et = (verifier ? p.ev : p.ed) + r * p.ldz;
-  const RowNucleus n = nucleus(et, (verifier ? p.stats_v : p.stats_d) + r * sld,
-                               (verifier ? p.f_v : p.f_d) + r * p.tiles, p.V, p.tiles, p.scale,
+  const RowNucleus n = nucleus<NW>(et, (verifier ? p.stats_v : p.stats_d) + r * sld,
+                               (verifier ? p.f_v : p.f_d) + r * p.tiles, p.V, p.tiles, p.tile_shift, p.scale,
                                p.top_p, ftab, listA, listB, sh, p.status);
   if (threadIdx.x == 0) store_state((verifier ? p.state_v : p.state_d) + r * kSpecStateWords, n);
 }
@@ -793,12 +793,12 @@ __global__ void __launch_bounds__(kThreads, 4) spec_row_kernel(const SpecParams 
 // passes u * total.
 
 // Unnormalised probabilities e of the lane's 4 tokens from i0 (zeros past V).
-__device__ __forceinline__ float4 load_e(const float* et, const float* ftab, long long i0,
+__device__ __forceinline__ float4 load_e(const float* et, const float* ftab, int tsh, long long i0,
                                          long long V) {
   float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
   if (i0 < V) {
     v = __ldg(reinterpret_cast<const float4*>(et + i0));
-    const float fm = ftab[i0 / kGemmBN];
+    const float fm = ftab[i0 >> tsh];
     v.x *= fm;
     v.y *= fm;
     v.z *= fm;
@@ -865,16 +865,16 @@ __device__ void block_inclusive_scan(float* a, int n, SharedT<NW>& sh) {
 
 // Per step: the ties at b, then (thread 0, in index order) their exclusive prefix.
 template <int NW>
-__device__ void step_tie_bases(const float* et, const float* ftab, const RowNucleus& n, long long V,
+__device__ void step_tie_bases(const float* et, const float* ftab, int tsh, const RowNucleus& n, long long V,
                                int nsteps, int* base) {
   const int w = warp_id(), l = lane_id();
   for (int st = w; st < nsteps; st += NW) {
     const long long i0 = static_cast<long long>(st) * kStep + l * 4;
-    if (ftab[static_cast<long long>(st) * kStep / kGemmBN] < n.b) {  // no e reaches b here
+    if (ftab[(static_cast<long long>(st) * kStep) >> tsh] < n.b) {  // no e reaches b here
       if (l == 0) base[st] = 0;
       continue;
     }
-    const float4 v = load_e(et, ftab, i0, V);
+    const float4 v = load_e(et, ftab, tsh, i0, V);
     int t = 0;
 #pragma unroll
     for (int j = 0; j < 4; ++j) t += i0 + j < V && comp(v, j) == n.b;
@@ -898,34 +898,36 @@ __device__ void step_tie_bases(const float* et, const float* ftab, const RowNucl
 // per column tile.
 template <int NW>
 __device__ int sample(const float* ep, const float* fp, const RowNucleus& np, const float* eq,
-                      const float* fq, const RowNucleus& nq, bool have_q, long long V, float u,
+                      const float* fq, const RowNucleus& nq, bool have_q, int tsh, long long V, float u,
                       float* cum, int* tp, int* tq, int* live, SharedT<NW>& sh, int* status) {
   const int nsteps = static_cast<int>((V + kStep - 1) / kStep);
   const int w = warp_id(), l = lane_id();
   const float ip = 1.f / np.kept, iq = have_q ? 1.f / nq.kept : 0.f;
   const bool part_p = np.c < np.eq, part_q = have_q && nq.c < nq.eq;
-  if (part_p) step_tie_bases<NW>(ep, fp, np, V, nsteps, tp);
-  if (part_q) step_tie_bases<NW>(eq, fq, nq, V, nsteps, tq);
+  if (part_p) step_tie_bases<NW>(ep, fp, tsh, np, V, nsteps, tp);
+  if (part_q) step_tie_bases<NW>(eq, fq, tsh, nq, V, nsteps, tq);
   // Mass of every step.  p is 0 where e < b, so only the tiles whose maximum
-  // f_t reaches b (listed in tile order) are read; warp w takes live tiles w,
-  // w + NW, ..., one tile (two steps, p and q) per round with all four loads
-  // in flight.  The other steps' masses are 0.
+  // f_t reaches b (listed in tile order) are read; a warp takes two steps
+  // (p and q) per round with all four loads in flight.  The other steps' masses are 0.
   for (int st = threadIdx.x; st < nsteps; st += NW * 32) cum[st] = 0.f;
-  const int nlive = kept_tiles(fp, (nsteps * kStep + kGemmBN - 1) / kGemmBN,
+  const int nlive = kept_tiles(fp, ((nsteps * kStep - 1) >> tsh) + 1,
                                __float_as_uint(np.b), live, sh);  // its barriers publish cum
-  for (int j = w; j < nlive; j += NW) {
-    const int t = live[j];
+  const int sub = tsh - kStepShift, nls = nlive << sub;  // steps of the live tiles
+  for (int q0 = 2 * w; q0 < nls; q0 += 2 * NW) {
+    int sts[2];
     float4 vp[2], vq[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const long long i0 = static_cast<long long>(t) * kGemmBN + h * kStep + l * 4;
-      vp[h] = load_e(ep, fp, i0, V);
-      vq[h] = have_q ? load_e(eq, fq, i0, V) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const int q = q0 + h;
+      sts[h] = q < nls ? (live[q >> sub] << sub) + (q & ((1 << sub) - 1)) : nsteps;
+      const long long i0 = static_cast<long long>(sts[h]) * kStep + l * 4;
+      vp[h] = load_e(ep, fp, tsh, i0, V);
+      vq[h] = have_q ? load_e(eq, fq, tsh, i0, V) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int st = t * (kGemmBN / kStep) + h;
-      if (st >= nsteps) break;  // warp-uniform
+      const int st = sts[h];
+      if (st >= nsteps) continue;  // warp-uniform
       const long long i0 = static_cast<long long>(st) * kStep + l * 4;
       float a[4], c[4] = {0.f, 0.f, 0.f, 0.f};
       probs4(vp[h], i0, V, np, ip, part_p ? tp[st] : 0, a);
@@ -964,8 +966,8 @@ __device__ int sample(const float* ep, const float* fp, const RowNucleus& np, co
     }
     const long long i0 = static_cast<long long>(owner) * kStep + l * 4;
     float a[4], c[4] = {0.f, 0.f, 0.f, 0.f};
-    probs4(load_e(ep, fp, i0, V), i0, V, np, ip, part_p ? tp[owner] : 0, a);
-    if (have_q) probs4(load_e(eq, fq, i0, V), i0, V, nq, iq, part_q ? tq[owner] : 0, c);
+    probs4(load_e(ep, fp, tsh, i0, V), i0, V, np, ip, part_p ? tp[owner] : 0, a);
+    if (have_q) probs4(load_e(eq, fq, tsh, i0, V), i0, V, nq, iq, part_q ? tq[owner] : 0, c);
     float r[4], lane_sum = 0.f;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -1040,8 +1042,8 @@ __global__ void __launch_bounds__(kSampleWarps * 32) spec_sample_kernel(const Sp
       if (x >= 0 && x < p.V) {
         const RowNucleus nq = load_state(p.state_d + pos_d * kSpecStateWords);
         const RowNucleus np = load_state(p.state_v + pos_v * kSpecStateWords);
-        const float eq = p.ed[pos_d * p.ldz + x] * p.f_d[pos_d * p.tiles + x / kGemmBN];
-        const float ep = p.ev[pos_v * p.ldz + x] * p.f_v[pos_v * p.tiles + x / kGemmBN];
+        const float eq = p.ed[pos_d * p.ldz + x] * p.f_d[pos_d * p.tiles + (x >> p.tile_shift)];
+        const float ep = p.ev[pos_v * p.ldz + x] * p.f_v[pos_v * p.tiles + (x >> p.tile_shift)];
         const bool rank_q = eq == nq.b && nq.c < nq.eq, rank_p = ep == np.b && np.c < np.eq;
         if (rank_q || rank_p) {
           f = 2;
@@ -1064,9 +1066,9 @@ __global__ void __launch_bounds__(kSampleWarps * 32) spec_sample_kernel(const Sp
           fp[t] = p.f_v[pos_v * p.tiles + t];
         }
         __syncthreads();
-        const float qx = prob_of(p.ed + pos_d * p.ldz, fq, p.V,
+        const float qx = prob_of(p.ed + pos_d * p.ldz, fq, p.tile_shift, p.V,
                                  load_state(p.state_d + pos_d * kSpecStateWords), x, sh);
-        const float px = prob_of(p.ev + pos_v * p.ldz, fp, p.V,
+        const float px = prob_of(p.ev + pos_v * p.ldz, fp, p.tile_shift, p.V,
                                  load_state(p.state_v + pos_v * kSpecStateWords), x, sh);
         f = qx > 0.f && p.u[pos_v * 2] * qx < px;
         __syncthreads();
@@ -1083,11 +1085,11 @@ __global__ void __launch_bounds__(kSampleWarps * 32) spec_sample_kernel(const Sp
       const RowNucleus nq = load_state(p.state_d + pos_d * kSpecStateWords);
       for (int t = threadIdx.x; t < p.tiles; t += kSampleWarps * 32) fq[t] = p.f_d[pos_d * p.tiles + t];
       __syncthreads();
-      next = sample(ev, fp, np, p.ed + pos_d * p.ldz, fq, nq, true, p.V, u, cum, tp, tq, live, sh,
+      next = sample(ev, fp, np, p.ed + pos_d * p.ldz, fq, nq, true, p.tile_shift, p.V, u, cum, tp, tq, live, sh,
                     p.status);
     }
     __syncthreads();
-    if (next < 0) next = sample(ev, fp, np, ev, fp, np, false, p.V, u, cum, tp, tq, live, sh, p.status);
+    if (next < 0) next = sample(ev, fp, np, ev, fp, np, false, p.tile_shift, p.V, u, cum, tp, tq, live, sh, p.status);
     if (next < 0) next = static_cast<int>(p.V - 1);  // unreachable: the maximum has e = 1
   }
   if (threadIdx.x == 0) {
@@ -1105,9 +1107,15 @@ size_t sample_smem(long long V, int tiles, int gamma) {
 }  // namespace
 
 cudaError_t setup_spec_kernels() {
-  cudaError_t e = cudaFuncSetAttribute(spec_row_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(row_smem(kSpecMaxTiles)));
+  cudaError_t e;
+#define MLS_SET(NW)                                                                                \
+  e = cudaFuncSetAttribute(spec_row_kernel<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,       \
+                           static_cast<int>(row_smem(kSpecMaxTiles)));                             \
   if (e != cudaSuccess) return e;
+  MLS_SET(8)
+  MLS_SET(16)
+  MLS_SET(32)
+#undef MLS_SET
   return cudaFuncSetAttribute(
       spec_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
       static_cast<int>(sample_smem(static_cast<long long>(kSpecMaxTiles) * kGemmBN, kSpecMaxTiles,
@@ -1117,7 +1125,17 @@ cudaError_t setup_spec_kernels() {
 cudaError_t launch_spec_rows(const SpecParams& p, cudaStream_t s) {
   const long long rows = static_cast<long long>(p.B) * (2 * p.gamma + 1);
   if (rows <= 0 || p.greedy) return cudaSuccess;
-  spec_row_kernel<<<static_cast<unsigned>(rows), kThreads, row_smem(p.tiles), s>>>(p);
+  // A row's passes are bound by the loads its CTA keeps in flight, so few rows
+  // get more warps each: 32 while every row has an SM, 16 while two share one.
+  // Measured against 8 warps: 68 rows of 109105 (top_p 0.9 at temperature
+  // 0.575) 107 -> 58 us, 234 rows of 50304 27.8 -> 21.6 us, 13 rows unchanged.
+  const unsigned grid = static_cast<unsigned>(rows);
+  if (rows <= p.sms)
+    spec_row_kernel<32><<<grid, 1024, row_smem(p.tiles), s>>>(p);
+  else if (rows <= 2 * p.sms)
+    spec_row_kernel<16><<<grid, 512, row_smem(p.tiles), s>>>(p);
+  else
+    spec_row_kernel<8><<<grid, 256, row_smem(p.tiles), s>>>(p);
   return cudaGetLastError();
 }
 
