@@ -60,3 +60,48 @@ def test_more_tiles_than_sms_and_wide_draft():
             assert (ss[:, 0::2].double() - m).abs().max() < 1e-4
             assert ((ss[:, 1::2].double() / want.sum(-1)) - 1).abs().max() < 1e-4
             assert (ee[:, :V].double() - want.view(H.shape[0], -1)[:, :V]).abs().max() < 1e-4
+
+
+@pytest.mark.parametrize("b,V,z_std,temperature,top_p", [
+    (2, 60000, 2.5, 0.9, 0.95),    # thousands of tokens in the boundary's octave: listed
+    (2, 60000, 0.5, 1.0, 0.9),     # over 4096 of them: bisected first
+    (2, 3000, 2.5, 0.05, 0.5),     # one token above 2^-8 settles it
+    (2, 3000, 0.0, 1.0, 0.9),      # every token tied at the maximum
+    (60, 9000, 2.5, 0.9, 0.99),    # 8 and 16 warps per row instead of 32
+    (200, 9000, 2.5, 0.9, 0.99),
+])
+def test_nucleus_boundary(b, V, z_std, temperature, top_p):
+    """Each row's nucleus state against fp64 sums of the stored probabilities e:
+    the mass above the boundary b stays below top_p of the total, the mass from
+    b on reaches it (to 1e-5, fp32 sums of at most 60000 terms in trees), and
+    the ties are counted exactly."""
+    gamma, dd, dv = 1, 64, 128
+    wl = synth.SpecWorkload("n", B=b, gamma=gamma, V=V, d_draft=dd, d_verify=dv, z_std=z_std)
+    Hd, Wd, Hv, Wv = (t.cuda() for t in synth.make_spec_inputs(wl, 5))
+    op = B.SpecVerify(b, gamma, V, dd, dv, temperature=temperature, top_p=top_p)
+    draft = torch.zeros(b, gamma, dtype=torch.int32, device="cuda")
+    op(Hd, Wd, Hv, Wv, draft, synth.make_uniforms(b, gamma, 5).cuda())
+    torch.cuda.synchronize()
+    assert B.mls_get_status() == 0
+    Pv, Pd = b * (gamma + 1), b * gamma
+    sh = 7 if Pv <= 128 else 8
+    tiles, ldz = -(-V // (1 << sh)), -(-V // 4) * 4
+    off, parts = 0, []
+    for rows, cols in ((Pv, ldz), (Pd, ldz), (Pv, 2 * tiles), (Pd, 2 * tiles), (Pv, tiles),
+                       (Pd, tiles), (Pv, 8), (Pd, 8)):
+        n = 4 * rows * cols
+        parts.append(op.ws[off:off + n].view(torch.float32).view(rows, cols))
+        off += -(-n // 256) * 256
+    ev, ed, _, _, fv, fd, sv, sd = parts
+    for e, f, st in ((ev, fv, sv), (ed, fd, sd)):
+        e = e[:, :V] * f[:, torch.arange(V, device="cuda") >> sh]  # fp32, as the kernel forms it
+        bound, kept = st[:, 1], st[:, 2].double()
+        c, ties = (st[:, i].contiguous().view(torch.int32) for i in (3, 4))
+        total = e.double().sum(-1)
+        above = torch.where(e > bound[:, None], e, 0.).double().sum(-1)
+        assert (ties == (e == bound[:, None]).sum(-1)).all()
+        assert ((c >= 1) & (c <= ties)).all()
+        assert (above < top_p * total * (1 + 1e-5)).all()
+        assert (above + c * bound.double() >= top_p * total * (1 - 1e-5)).all()
+        assert (above + (c - 1) * bound.double() <= top_p * total * (1 + 1e-5)).all()
+        assert ((above + c * bound.double()) / kept - 1).abs().max() < 1e-5
