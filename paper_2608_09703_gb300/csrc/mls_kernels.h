@@ -338,7 +338,7 @@ __host__ __device__ inline int merge_warps_per_octet(int nparts) {
 __host__ __device__ inline int merge_tokens_per_block(int nparts) {
   return 8 * (8 / merge_warps_per_octet(nparts));
 }
-constexpr int kEvalMergeTokens = 128;  // tokens per evaluation-merge block: one thread per token
+constexpr int kEvalMergeTokens = 32;  // tokens per evaluation-merge block: one per lane
 
 // Launchers (return the cudaError_t of the launch).
 cudaError_t launch_head_fwd(const HeadParams& p, bool tf32, bool tau_one, cudaStream_t s);
