@@ -667,7 +667,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kHeadThreads, 1)
   if (warp >= kHeadEpiWarps) {
     regs_decrease<kHeadCtlRegs>();
     if (warp == kHeadEpiWarps) {
-      if (lane == 0) eval_producer<kTF32, kM>(p, base, row_base, rank, split, abort_flag);
+      if (lane == 0) {
+        eval_producer<kTF32, kM>(p, base, row_base, rank, split, abort_flag);
+        chain_trigger();
+      }
     } else if (warp == kHeadEpiWarps + 1) {
       if (lane == 0 && rank == 0) {
         if constexpr (eval_slotted(kM))
@@ -728,6 +731,8 @@ __global__ void __launch_bounds__(kEvalMergeWarps * 32)
   const float L1 = 1.4426950408889634f;
   const bool live = t < T;
   const float* P = p.part + (live ? t : 0);
+  chain_trigger();
+  chain_wait();
   float mm[kM];
 #pragma unroll
   for (int s = 0; s < kM; ++s) mm[s] = -INFINITY;
@@ -820,10 +825,12 @@ __global__ void __launch_bounds__(kEvalMergeWarps * 32)
 constexpr int kEvalFinalThreads = 256;
 
 __global__ void __launch_bounds__(kEvalFinalThreads)
-    eval_final_kernel(const double* __restrict__ acc, const long long* __restrict__ cnt, int n,
+    eval_final_kernel(const double* acc, const long long* cnt, int n,
                       int M, float* pair_stats) {
   __shared__ double sh[kEvalFinalThreads / 32];
   const int q = blockIdx.x / (M * M), e = blockIdx.x % (M * M);
+  chain_trigger();
+  chain_wait();
   double c = 0.0, s = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     c += static_cast<double>(cnt[i]);
@@ -858,18 +865,17 @@ cudaError_t launch_eval(const EvalParams& p, bool tf32, cudaStream_t s) {
 cudaError_t launch_eval_merge(const EvalMergeParams& p, int blocks, cudaStream_t s) {
   if (blocks <= 0) return cudaSuccess;
   switch (p.M) {
-    case 1: eval_merge_kernel<1><<<blocks, kEvalMergeWarps * 32, 0, s>>>(p); break;
-    case 2: eval_merge_kernel<2><<<blocks, kEvalMergeWarps * 32, 0, s>>>(p); break;
-    case 3: eval_merge_kernel<3><<<blocks, kEvalMergeWarps * 32, 0, s>>>(p); break;
-    default: eval_merge_kernel<4><<<blocks, kEvalMergeWarps * 32, 0, s>>>(p); break;
+    case 1: return launch_chained(eval_merge_kernel<1>, dim3(blocks), dim3(kEvalMergeWarps * 32), 0, s, p);
+    case 2: return launch_chained(eval_merge_kernel<2>, dim3(blocks), dim3(kEvalMergeWarps * 32), 0, s, p);
+    case 3: return launch_chained(eval_merge_kernel<3>, dim3(blocks), dim3(kEvalMergeWarps * 32), 0, s, p);
+    default: return launch_chained(eval_merge_kernel<4>, dim3(blocks), dim3(kEvalMergeWarps * 32), 0, s, p);
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_eval_final(const double* block_acc, const long long* block_cnt, int nblocks,
                               int M, float* pair_stats, cudaStream_t s) {
-  eval_final_kernel<<<2 * M * M, kEvalFinalThreads, 0, s>>>(block_acc, block_cnt, nblocks, M, pair_stats);
-  return cudaGetLastError();
+  return launch_chained(eval_final_kernel, dim3(2 * M * M), dim3(kEvalFinalThreads), 0, s, block_acc,
+                        block_cnt, nblocks, M, pair_stats);
 }
 
 cudaError_t setup_eval_kernels() {

@@ -555,7 +555,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
   const uint32_t tmem = *tmem_slot;
 
   if (warp == kGemmEpiWarps) {
-    if (lane == 0) gemm_producer<kTF32, kAMode, kBMN>(p, base, rank, abort_flag);
+    if (lane == 0) {
+      chain_wait();  // dL/dz is complete (the epilogue's stores follow from these loads)
+      gemm_producer<kTF32, kAMode, kBMN>(p, base, rank, abort_flag);
+      chain_trigger();
+    }
   } else if (warp == kGemmEpiWarps + 1) {
     if (lane == 0 && rank == 0) gemm_mma<kTF32, kAMode, kBMN>(p, base, tmem, abort_flag);
     __syncwarp();
@@ -571,23 +575,28 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
   }
 }
 
-template <int kAMode, bool kBMN, bool kStats>
-cudaError_t launch(const GemmParams& p, bool tf32, int grid, cudaStream_t s) {
-  if (p.total_tiles <= 0 || grid <= 0) return cudaSuccess;
-  if (tf32)
-    gemm_kernel<true, kAMode, kBMN, kStats><<<grid, kGemmThreads, kGemmSmem, s>>>(p);
-  else
-    gemm_kernel<false, kAMode, kBMN, kStats><<<grid, kGemmThreads, kGemmSmem, s>>>(p);
-  return cudaGetLastError();
-}
-
 }  // namespace
 
+// The verify step's first kernel.
 cudaError_t launch_gemm_stats(const GemmParams& p, bool tf32, int grid, cudaStream_t s) {
-  return launch<0, false, true>(p, tf32, grid, s);
+  if (p.total_tiles <= 0 || grid <= 0) return cudaSuccess;
+  if (tf32)
+    gemm_kernel<true, 0, false, true><<<grid, kGemmThreads, kGemmSmem, s>>>(p);
+  else
+    gemm_kernel<false, 0, false, true><<<grid, kGemmThreads, kGemmSmem, s>>>(p);
+  return cudaGetLastError();
 }
 cudaError_t launch_gemm_mixed(const GemmParams& p, bool tf32, int grid, cudaStream_t s) {
-  return launch<2, true, false>(p, tf32, grid, s);
+  if (p.total_tiles <= 0 || grid <= 0) return cudaSuccess;
+  if (!p.chained) {
+    if (tf32)
+      gemm_kernel<true, 2, true, false><<<grid, kGemmThreads, kGemmSmem, s>>>(p);
+    else
+      gemm_kernel<false, 2, true, false><<<grid, kGemmThreads, kGemmSmem, s>>>(p);
+    return cudaGetLastError();
+  }
+  return launch_chained(tf32 ? gemm_kernel<true, 2, true, false> : gemm_kernel<false, 2, true, false>,
+                        dim3(grid), dim3(kGemmThreads), kGemmSmem, s, p);
 }
 
 // How many CTA pairs of the GEMM kernel can be resident at once (GPCs with an

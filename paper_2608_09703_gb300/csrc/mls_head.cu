@@ -587,7 +587,8 @@ __device__ __forceinline__ void bwd_epilogue(const HeadParams& p, uint32_t base,
   const bool row_ok = row < p.T;
   const int y = row_ok ? __ldg(p.y + row) : -1;
   const bool valid = row_ok && y >= 0 && y < p.V;
-  const float inv_n = *p.inv_n;
+  chain_wait();  // 1/N is there, and the GEMM of the group before has read its dL/dz
+  const float inv_n = *reinterpret_cast<const volatile float*>(p.inv_n);
   const uint32_t tl = tmem + (static_cast<uint32_t>(quad * 32) << 16) + static_cast<uint32_t>(half * 128);
   const float L1 = p.L1, Lt = p.Ltau;
   const long long MT = static_cast<long long>(p.M) * p.T;
@@ -715,7 +716,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kHeadThreads, 1)
   if (warp >= kHeadEpiWarps) {
     regs_decrease<kHeadCtlRegs>();
     if (warp == kHeadEpiWarps) {
-      if (lane == 0) head_producer<kTF32>(p, base, row_base, rank, split, abort_flag);
+      if (lane == 0) {
+        head_producer<kTF32>(p, base, row_base, rank, split, abort_flag);
+        chain_trigger();
+      }
     } else if (warp == kHeadEpiWarps + 1) {
       if (lane == 0 && rank == 0) head_mma<kTF32>(p, base, tmem, split, abort_flag);
       __syncwarp();
@@ -737,19 +741,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kHeadThreads, 1)
   }
 }
 
+// The forward is its call's first kernel, the backward follows the token count.
+template <int kMode, bool kTF32, bool kTauOne>
+cudaError_t launch_mode(const HeadParams& p, int grid, cudaStream_t s) {
+  if constexpr (kMode == kModeBwd)
+    return launch_chained(head_kernel<kMode, kTF32, kTauOne>, dim3(grid), dim3(kHeadThreads), kHeadSmem, s, p);
+  head_kernel<kMode, kTF32, kTauOne><<<grid, kHeadThreads, kHeadSmem, s>>>(p);
+  return cudaGetLastError();
+}
+
 template <int kMode>
 cudaError_t launch_head(const HeadParams& p, bool tf32, bool tau_one, cudaStream_t s) {
   const int grid = 2 * p.ntt * p.S;  // CTA pairs
   if (grid <= 0) return cudaSuccess;
-  const dim3 g(grid), b(kHeadThreads);
-  if (tf32) {
-    if (tau_one) head_kernel<kMode, true, true><<<g, b, kHeadSmem, s>>>(p);
-    else head_kernel<kMode, true, false><<<g, b, kHeadSmem, s>>>(p);
-  } else {
-    if (tau_one) head_kernel<kMode, false, true><<<g, b, kHeadSmem, s>>>(p);
-    else head_kernel<kMode, false, false><<<g, b, kHeadSmem, s>>>(p);
-  }
-  return cudaGetLastError();
+  if (tf32) return tau_one ? launch_mode<kMode, true, true>(p, grid, s) : launch_mode<kMode, true, false>(p, grid, s);
+  return tau_one ? launch_mode<kMode, false, true>(p, grid, s) : launch_mode<kMode, false, false>(p, grid, s);
 }
 
 template <int kMode>

@@ -9,6 +9,24 @@
 
 namespace mls {
 
+// Launches a kernel that may start before the stream's previous kernel has
+// completed (see chain_wait).
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                           const A&... args) {
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 constexpr int kMaxModels = 4;
 
 // ------------------------------------------------------------------ head kernels
@@ -169,6 +187,7 @@ struct GemmParams {
   int two_class;
   int n_long;
   int catchup;
+  int chained;                   // launch_gemm_mixed: may start before its predecessor has completed
 };
 
 // ------------------------------------------------------------------ pairwise evaluation

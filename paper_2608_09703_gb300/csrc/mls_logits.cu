@@ -257,6 +257,7 @@ __global__ void __launch_bounds__(kThreads, 1) logits_kernel(const __grid_consta
         for (int s = 0; s < stages; ++s)
           if ((filled >> s) & 1u)
             mbar_wait_drain(smem_u32(&sh->full[s]), (lastpar >> s) & 1u, kDrainNs, p.status);
+      chain_trigger();
     }
   } else if (warp == kEpi + 1) {
     if (lane == 0) {

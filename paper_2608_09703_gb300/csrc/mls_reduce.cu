@@ -64,6 +64,8 @@ __global__ void __launch_bounds__(kMergeWarps * 32, 4) merge_kernel(const __grid
   const long long PS = kPartFields * MT;  // stride between partials
   const int tc = p.teacher;
   const int k0 = 4 * ww + grp;
+  chain_trigger();
+  chain_wait();
 
   // ---- pass 1: row maxima of every sub-model
   float mx[kMaxModels];
@@ -258,9 +260,11 @@ __global__ void __launch_bounds__(kMergeWarps * 32, 4) merge_kernel(const __grid
 constexpr int kFinalThreads = 256;
 
 __global__ void __launch_bounds__(kFinalThreads)
-    final_kernel(const double* __restrict__ bsum, const long long* __restrict__ bcnt, int n,
+    final_kernel(const double* bsum, const long long* bcnt, int n,
                  float* loss) {
   __shared__ double sh[kFinalThreads / 32];
+  chain_trigger();
+  chain_wait();
   double s = 0.0, c = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     s += bsum[i];
@@ -278,6 +282,8 @@ constexpr int kSplitSumThreads = 256;
 
 __global__ void __launch_bounds__(kSplitSumThreads)
     split_sum_kernel(const __grid_constant__ SplitSumParams p) {
+  chain_trigger();
+  chain_wait();
   const int m = blockIdx.y;
   const long long n4 = p.n4[m], s4 = p.stride / 4;
   const float4* part = reinterpret_cast<const float4*>(p.part[m]);
@@ -302,6 +308,7 @@ constexpr int kCountThreads = 1024;
 __global__ void __launch_bounds__(kCountThreads)
     count_kernel(const int* __restrict__ y, long long T, long long V, float* inv_n, int* status) {
   __shared__ double sh[kCountThreads / 32];
+  chain_trigger();
   double c = 0.0;
   bool bad = false;
   for (long long i = threadIdx.x; i < T; i += blockDim.x) {
@@ -319,17 +326,15 @@ __global__ void __launch_bounds__(kCountThreads)
 cudaError_t launch_merge(const MergeParams& p, int blocks, cudaStream_t s) {
   if (blocks <= 0) return cudaSuccess;
   switch (merge_warps_per_octet(p.nparts)) {
-    case 1: merge_kernel<1><<<blocks, kMergeWarps * 32, 0, s>>>(p); break;
-    case 2: merge_kernel<2><<<blocks, kMergeWarps * 32, 0, s>>>(p); break;
-    default: merge_kernel<8><<<blocks, kMergeWarps * 32, 0, s>>>(p); break;
+    case 1: return launch_chained(merge_kernel<1>, dim3(blocks), dim3(kMergeWarps * 32), 0, s, p);
+    case 2: return launch_chained(merge_kernel<2>, dim3(blocks), dim3(kMergeWarps * 32), 0, s, p);
+    default: return launch_chained(merge_kernel<8>, dim3(blocks), dim3(kMergeWarps * 32), 0, s, p);
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_final(const double* block_sum, const long long* block_cnt, int nblocks,
                          float* loss, cudaStream_t s) {
-  final_kernel<<<1, kFinalThreads, 0, s>>>(block_sum, block_cnt, nblocks, loss);
-  return cudaGetLastError();
+  return launch_chained(final_kernel, dim3(1), dim3(kFinalThreads), 0, s, block_sum, block_cnt, nblocks, loss);
 }
 
 cudaError_t launch_split_sum(const SplitSumParams& p, cudaStream_t s) {
@@ -338,8 +343,7 @@ cudaError_t launch_split_sum(const SplitSumParams& p, cudaStream_t s) {
   if (most <= 0) return cudaSuccess;
   const long long blocks = (most + kSplitSumThreads - 1) / kSplitSumThreads;
   const dim3 grid(static_cast<unsigned>(blocks < 4096 ? blocks : 4096), p.nprob);
-  split_sum_kernel<<<grid, kSplitSumThreads, 0, s>>>(p);
-  return cudaGetLastError();
+  return launch_chained(split_sum_kernel, grid, dim3(kSplitSumThreads), 0, s, p);
 }
 
 cudaError_t launch_count(const int* y, long long T, long long V, float* inv_n, int* status,

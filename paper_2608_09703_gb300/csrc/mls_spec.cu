@@ -875,6 +875,8 @@ __global__ void __launch_bounds__(NW * 32, 32 / NW) spec_row_kernel(const SpecPa
   static_assert(kFinish <= NW * 32, "one candidate per thread in the exact finish");
   extern __shared__ __align__(16) float smem[];
   __shared__ SharedT<NW> sh;
+  chain_trigger();
+  chain_wait();
   const int tiles_pad = (p.tiles + 3) / 4 * 4;
   float* ftab = smem;
   float* listA = smem + tiles_pad;
@@ -1117,6 +1119,8 @@ __device__ int row_argmax(const float* st, int tiles, SharedT<NW>& sh) {
 __global__ void __launch_bounds__(kSampleWarps * 32) spec_sample_kernel(const SpecParams p) {
   extern __shared__ __align__(16) float smem[];
   __shared__ SharedT<kSampleWarps> sh;
+  chain_trigger();
+  chain_wait();
   const int b = blockIdx.x, G1 = p.gamma + 1;
   const long long sld = 2LL * p.tiles;
   int k = 0, next = -1;
@@ -1235,19 +1239,15 @@ cudaError_t launch_spec_rows(const SpecParams& p, cudaStream_t s) {
   // Measured against 8 warps: 68 rows of 109105 (top_p 0.9 at temperature
   // 0.575) 107 -> 58 us, 234 rows of 50304 27.8 -> 21.6 us, 13 rows unchanged.
   const unsigned grid = static_cast<unsigned>(rows);
-  if (rows <= p.sms)
-    spec_row_kernel<32><<<grid, 1024, row_smem(p.tiles, 32), s>>>(p);
-  else if (rows <= 2 * p.sms)
-    spec_row_kernel<16><<<grid, 512, row_smem(p.tiles, 16), s>>>(p);
-  else
-    spec_row_kernel<8><<<grid, 256, row_smem(p.tiles, 8), s>>>(p);
-  return cudaGetLastError();
+  if (rows <= p.sms) return launch_chained(spec_row_kernel<32>, dim3(grid), dim3(1024), row_smem(p.tiles, 32), s, p);
+  if (rows <= 2 * p.sms) return launch_chained(spec_row_kernel<16>, dim3(grid), dim3(512), row_smem(p.tiles, 16), s, p);
+  return launch_chained(spec_row_kernel<8>, dim3(grid), dim3(256), row_smem(p.tiles, 8), s, p);
 }
 
 cudaError_t launch_spec_sample(const SpecParams& p, cudaStream_t s) {
   if (p.B <= 0) return cudaSuccess;
-  spec_sample_kernel<<<p.B, kSampleWarps * 32, p.greedy ? 0 : sample_smem(p.V, p.tiles, p.gamma), s>>>(p);
-  return cudaGetLastError();
+  return launch_chained(spec_sample_kernel, dim3(p.B), dim3(kSampleWarps * 32),
+                        p.greedy ? 0 : sample_smem(p.V, p.tiles, p.gamma), s, p);
 }
 
 }  // namespace mls
