@@ -624,9 +624,6 @@ extern "C" int mls_head_loss_bwd(const mls_problem* p, const void* const* H, con
   for (int m = 0; m < p->M; ++m) hp.coef[m] = grad_scale * (p->w ? p->w[m] : 1.0f);
   hp.one_minus_alpha = 1.0f - p->alpha;
   hp.alpha_over_tau = p->alpha / p->tau;
-  hp.G = G;
-  hp.g_pitch = pl.group;
-  hp.g_model_stride = p->T * pl.group;
 
   // dW reads A = G viewed M-major and B = H viewed N-major, dH reads A = G
   // K-major and B = W viewed N-major, all in place.
@@ -636,10 +633,9 @@ extern "C" int mls_head_loss_bwd(const mls_problem* p, const void* const* H, con
   const CUtensorMapSwizzle mn_swizzle =
       tf32 ? CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B : CU_TENSOR_MAP_SWIZZLE_128B;
   for (int m = 0; m < p->M; ++m) {
-    const void* Gm = static_cast<const char*>(G) + static_cast<size_t>(pl.elt) * hp.g_model_stride * m;
-    // the backward head kernel's TMA stores of 32x32 dL/dz chunks (bf16 only)
-    if (!tf32 && encode(&hp.mapG[m], Gm, 2, pl.group, p->T, pl.group, 32, 32,
-                        CU_TENSOR_MAP_SWIZZLE_64B))
+    const void* Gm = static_cast<const char*>(G) + static_cast<size_t>(pl.elt) * p->T * pl.group * m;
+    // the backward head kernel's TMA stores of dL/dz
+    if (encode(&hp.mapG[m], Gm, pl.elt, pl.group, p->T, pl.group, KE / 2, 32, CU_TENSOR_MAP_SWIZZLE_64B))
       return MLS_ERR_CUDA;
     if (encode(&gh.mapA[m], Gm, pl.elt, pl.group, p->T, pl.group, KE, kGemmBM) ||
         encode(&gw.mapA[m], Gm, pl.elt, pl.group, p->T, pl.group, KE, KE, mn_swizzle) ||

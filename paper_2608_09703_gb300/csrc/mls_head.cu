@@ -451,66 +451,59 @@ __device__ __forceinline__ void fwd_epilogue(const HeadParams& p, uint32_t base,
 }
 
 // ------------------------------------------------------------------ backward epilogue
-template <bool kTF32>
-__device__ __forceinline__ void store_chunk(void* dst, const float (&g)[32]) {
-  if constexpr (kTF32) {
-    float4* d = reinterpret_cast<float4*>(dst);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) d[i] = make_float4(g[4 * i], g[4 * i + 1], g[4 * i + 2], g[4 * i + 3]);
-  } else {
-    uint4* d = reinterpret_cast<uint4*>(dst);
-    uint32_t w[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      __nv_bfloat162 h = __floats2bfloat162_rn(g[2 * i], g[2 * i + 1]);
-      w[i] = *reinterpret_cast<uint32_t*>(&h);
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) d[i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
-  }
-}
-
-// Where one warp's 32x32 chunk of dL/dz goes.  bf16: staged in this warp's
-// shared-memory buffers (64B swizzle: 16-byte piece j of row r sits at piece
-// j ^ ((r >> 1) & 3)) and written by a TMA store; fp32: direct global stores.
+// Where one warp's 32x32 chunk of dL/dz goes: staged in this warp's two
+// shared-memory buffers of 32 rows x 64 bytes (64B swizzle: 16-byte piece j of
+// row r sits at piece j ^ ((r >> 1) & 3)) and written by TMA stores, a bf16 chunk
+// as one box, an fp32 one as two of 16 columns.  (fp32 stored by each thread to
+// its own row took the backward head of 2048 tokens, d = (768, 1536), V = 32768
+// 444 us, now 391; 256 tokens, d = (128,
+// 256), V = 1024: 22 and 17 us with the events around them.)
 struct GOut {
-  const CUtensorMap* map;  // bf16 TMA store map of this sub-model
+  const CUtensorMap* map;  // TMA store map of this sub-model
   uint32_t stage;          // this warp's two staging buffers
-  uint32_t* count;         // chunks issued by this warp (buffer parity)
+  uint32_t* count;         // boxes issued by this warp (buffer parity)
   int row0;                // first token row of the warp
-  char* gdst;              // fp32: this thread's row pointer at the unit's first column
-  bool row_ok;
 };
+
+// One box: this lane's row of it as 64 bytes.
+__device__ __forceinline__ void put_box(const GOut& o, int col, const uint32_t (&w)[16], int lane) {
+  const uint32_t buf = o.stage + ((*o.count) & 1u) * kHeadStageChunk;
+  if (lane == 0) bulk_wait_read<1>();  // the store that last used this buffer has read it
+  __syncwarp();
+  const uint32_t rowaddr = buf + lane * 64;
+  const uint32_t sw = (lane >> 1) & 3;
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    st_shared_v4(rowaddr + ((j ^ sw) << 4), w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+  fence_proxy_async_smem();
+  __syncwarp();
+  if (lane == 0) {
+    // dL/dz is read back by the GEMMs only after the whole launch, so its
+    // lines are the first to go from L2, ahead of the band's H and W.
+    tma_store_2d_hint(o.map, buf, col, o.row0, l2_policy_evict_first());
+    bulk_commit();
+  }
+  *o.count += 1;
+}
 
 template <bool kTF32>
 __device__ __forceinline__ void put_chunk(const GOut& o, int gcol, int ch, const float (&g)[32],
                                           int lane) {
+  uint32_t w[16];
   if constexpr (kTF32) {
-    if (o.row_ok) store_chunk<true>(o.gdst + ch * 32 * 4, g);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) w[i] = __float_as_uint(g[16 * h + i]);
+      put_box(o, gcol + ch * 32 + 16 * h, w, lane);
+    }
   } else {
-    const uint32_t buf = o.stage + ((*o.count) & 1u) * kHeadStageChunk;
-    if (lane == 0) bulk_wait_read<1>();  // the store that last used this buffer has read it
-    __syncwarp();
-    uint32_t w[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       __nv_bfloat162 h = __floats2bfloat162_rn(g[2 * i], g[2 * i + 1]);
       w[i] = *reinterpret_cast<uint32_t*>(&h);
     }
-    const uint32_t rowaddr = buf + lane * 64;
-    const uint32_t sw = (lane >> 1) & 3;
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      st_shared_v4(rowaddr + ((j ^ sw) << 4), w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
-    fence_proxy_async_smem();
-    __syncwarp();
-    if (lane == 0) {
-      // dL/dz is read back by the GEMMs only after the whole launch, so its
-      // lines are the first to go from L2, ahead of the band's H and W.
-      tma_store_2d_hint(o.map, buf, gcol + ch * 32, o.row0, l2_policy_evict_first());
-      bulk_commit();
-    }
-    *o.count += 1;
+    put_box(o, gcol + ch * 32, w, lane);
   }
 }
 
@@ -581,7 +574,6 @@ template <bool kTauOne, bool kTF32>
 __device__ __forceinline__ void bwd_epilogue(const HeadParams& p, uint32_t base, uint32_t tmem,
                                              int row_base, int split, int warp, int lane,
                                              volatile int* abort_flag) {
-  constexpr int kElt = kTF32 ? 4 : 2;
   const int quad = warp & 3, half = warp >> 2;
   const long long row = static_cast<long long>(row_base) + quad * 32 + lane;
   const bool row_ok = row < p.T;
@@ -602,9 +594,7 @@ __device__ __forceinline__ void bwd_epilogue(const HeadParams& p, uint32_t base,
   uint32_t nchunks = 0;
   const uint32_t stage = base + HeadSmem::kStage + static_cast<uint32_t>(warp) * 2 * kHeadStageChunk;
   const int row0 = row_base + quad * 32;
-  const GOut oT{&p.mapG[t], stage, &nchunks, row0,
-                static_cast<char*>(p.G) + (static_cast<long long>(t) * p.g_model_stride + rr * p.g_pitch) * kElt,
-                row_ok};
+  const GOut oT{&p.mapG[t], stage, &nchunks, row0};
 
   float a1[kStud], a2[kStud], b1[kStud], bt[kStud];
   int ms[kStud];
@@ -630,12 +620,10 @@ __device__ __forceinline__ void bwd_epilogue(const HeadParams& p, uint32_t base,
     if (!epi_acquire(p, base, acc, acc_par, abort_flag)) break;
     {
       const uint32_t ta = tl + acc * kHeadBN;
-      GOut o = oT;
-      o.gdst += static_cast<long long>(gcol) * kElt;
       if (nvalid == 128)
-        bwd_teacher<false, kTauOne, kTF32>(ta, 128, yl, L1, Lt, bT1, bTt, cT, q, o, gcol, lane);
+        bwd_teacher<false, kTauOne, kTF32>(ta, 128, yl, L1, Lt, bT1, bTt, cT, q, oT, gcol, lane);
       else
-        bwd_teacher<true, kTauOne, kTF32>(ta, nvalid, yl, L1, Lt, bT1, bTt, cT, q, o, gcol, lane);
+        bwd_teacher<true, kTauOne, kTF32>(ta, nvalid, yl, L1, Lt, bT1, bTt, cT, q, oT, gcol, lane);
     }
     epi_release(base, acc, acc_par, lane);
 
@@ -648,10 +636,7 @@ __device__ __forceinline__ void bwd_epilogue(const HeadParams& p, uint32_t base,
           break;
         }
         const uint32_t ta = tl + acc * kHeadBN;
-        const GOut o{&p.mapG[ms[j]], stage, &nchunks, row0,
-                     static_cast<char*>(p.G) +
-                         (static_cast<long long>(ms[j]) * p.g_model_stride + rr * p.g_pitch + gcol) * kElt,
-                     row_ok};
+        const GOut o{&p.mapG[ms[j]], stage, &nchunks, row0};
         if (nvalid == 128)
           bwd_student<false, kTauOne, kTF32>(ta, 128, yl, L1, Lt, b1[j], bt[j], a1[j], a2[j], q,
                                              o, gcol, lane);
@@ -664,7 +649,7 @@ __device__ __forceinline__ void bwd_epilogue(const HeadParams& p, uint32_t base,
     if (aborted) break;
   }
   // Every staged store has finished before the CTA's shared memory goes away.
-  if (!kTF32 && lane == 0) bulk_wait_all();
+  if (lane == 0) bulk_wait_all();
   __syncwarp();
 }
 

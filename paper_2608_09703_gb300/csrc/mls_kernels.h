@@ -50,8 +50,8 @@ static_assert(2 * 128 * kHeadEpiRegs + 128 * kHeadCtlRegs == kHeadThreads * kHea
               "register reallocation must add up to the launch allocation");
 constexpr uint32_t kHeadABytes = kHeadBM * 128;
 constexpr uint32_t kHeadBBytes = kHeadBHalf * 128;
-// Backward: each epilogue warp stages its dL/dz chunks (32 tokens x 32 bf16
-// columns, 2 KB, 64B-swizzled) in two buffers and writes them with TMA stores.
+// Backward: each epilogue warp stages its dL/dz chunks (32 tokens x 64 bytes of
+// columns, 64B-swizzled) in two buffers and writes them with TMA stores.
 constexpr uint32_t kHeadStageChunk = 32 * 64;
 constexpr uint32_t kHeadStaging = kHeadEpiWarps * 2 * kHeadStageChunk;
 constexpr uint32_t kHeadSmem = kHeadStages * (kHeadABytes + kHeadBBytes) + kHeadStaging + 1024 + 1024;
@@ -105,10 +105,7 @@ struct HeadParams {
   float coef[kMaxModels];        // grad_scale * w_m
   float one_minus_alpha;         // (1 - alpha)
   float alpha_over_tau;          // alpha / tau
-  CUtensorMap mapG[kMaxModels];  // G_m [T, g_pitch] bf16, box {32, 32}, 64B swizzle (TMA store)
-  void* G;                       // [M][T][g_pitch] bf16 (fp32 for fp32 inputs)
-  long long g_model_stride;      // elements
-  long long g_pitch;             // elements per token row
+  CUtensorMap mapG[kMaxModels];  // G_m [T, group] bf16 (fp32), box {64 bytes, 32}, 64B swizzle (TMA store)
   long long g_col0;              // vocabulary column of the group's first column
 };
 
