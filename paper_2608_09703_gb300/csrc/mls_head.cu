@@ -456,8 +456,7 @@ __device__ __forceinline__ void fwd_epilogue(const HeadParams& p, uint32_t base,
 // row r sits at piece j ^ ((r >> 1) & 3)) and written by TMA stores, a bf16 chunk
 // as one box, an fp32 one as two of 16 columns.  (fp32 stored by each thread to
 // its own row took the backward head of 2048 tokens, d = (768, 1536), V = 32768
-// 444 us, now 391; 256 tokens, d = (128,
-// 256), V = 1024: 22 and 17 us with the events around them.)
+// 444 us, now 391; of 256 tokens, d = (128, 256), V = 1024 22 us, now 17.)
 struct GOut {
   const CUtensorMap* map;  // TMA store map of this sub-model
   uint32_t stage;          // this warp's two staging buffers
