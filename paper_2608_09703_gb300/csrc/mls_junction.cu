@@ -137,8 +137,13 @@ __device__ __forceinline__ FwdRow fwd_row(const JunctionParams& p, long long t) 
           x + (p.embed_first ? de : 0), x + (p.embed_first ? 0 : p.d_prev)};
 }
 
-// kR > 0: both segments fit kR cached vectors per lane; kR == 0: streaming.
-template <typename E, int kR>
+// kRo, kRe > 0: the segments fit kRo and kRe cached vectors per lane; 0: streaming.
+// The two are separate because registers bound the rows in flight per SM: with
+// the larger one for both, 2048 + 1024 bf16 channels took 157 registers in the
+// backward (12 rows per SM), now 123 (16): at 65536 tokens 186 -> 170 us; both
+// junctions of the 3-level suite at 8192 tokens, forward and backward, 81.2 -> 78.8
+// us; 192 + 1296 channels at 8000 tokens 30.3 -> 24.6 us.
+template <typename E, int kRo, int kRe>
 __global__ void __launch_bounds__(32 * kRowsPerBlock) junction_fwd_kernel(const JunctionParams p) {
   constexpr int N = Vec<E>::N;
   const long long t = static_cast<long long>(blockIdx.x) * kRowsPerBlock + (threadIdx.x >> 5);
@@ -149,16 +154,16 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock) junction_fwd_kernel(const 
   const E* e = static_cast<const E*>(r.e);
   E* xo = static_cast<E*>(r.xo);
   E* xe = static_cast<E*>(r.xe);
-  if constexpr (kR > 0) {
-    uint4 vo[kR], ve[kR];
-    load_seg<E, kR>(o, p.d_prev, lane, vo);
-    load_seg<E, kR>(e, r.de, lane, ve);
-    const float no = sqrtf(warp_sum(sumsq_cached<E, kR>(vo)));
-    const float ne = sqrtf(warp_sum(sumsq_cached<E, kR>(ve)));
+  if constexpr (kRo > 0) {
+    uint4 vo[kRo], ve[kRe];
+    load_seg<E, kRo>(o, p.d_prev, lane, vo);
+    load_seg<E, kRe>(e, r.de, lane, ve);
+    const float no = sqrtf(warp_sum(sumsq_cached<E, kRo>(vo)));
+    const float ne = sqrtf(warp_sum(sumsq_cached<E, kRe>(ve)));
     const float s = no > 0.f ? ne / no : 0.f;
     keep_packed(vo);
 #pragma unroll
-    for (int j = 0; j < kR; ++j) {
+    for (int j = 0; j < kRo; ++j) {
       const int k = (j * 32 + lane) * N;
       if (k < p.d_prev) {
         float f[N];
@@ -167,6 +172,10 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock) junction_fwd_kernel(const 
         for (int i = 0; i < N; ++i) f[i] *= s;
         st16(xo + k, Vec<E>::pack(f));
       }
+    }
+#pragma unroll
+    for (int j = 0; j < kRe; ++j) {
+      const int k = (j * 32 + lane) * N;
       if (k < r.de) st16(xe + k, ve[j]);
     }
   } else {
@@ -184,7 +193,7 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock) junction_fwd_kernel(const 
   }
 }
 
-template <typename E, int kR>
+template <typename E, int kRo, int kRe>
 __global__ void __launch_bounds__(32 * kRowsPerBlock) junction_bwd_kernel(const JunctionParams p) {
   constexpr int N = Vec<E>::N;
   const long long t = static_cast<long long>(blockIdx.x) * kRowsPerBlock + (threadIdx.x >> 5);
@@ -199,15 +208,15 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock) junction_bwd_kernel(const 
   E* d_o = static_cast<E*>(p.d_o) + t * p.d_prev;
   E* d_e = static_cast<E*>(p.d_e) + t * de;
   float oo = 0.f, dot = 0.f, ee;
-  if constexpr (kR > 0) {
+  if constexpr (kRo > 0) {
     // Every input vector of the row is loaded at once and stays in registers.
-    uint4 vo[kR], vg[kR], ve[kR], vge[kR];
-    load_seg<E, kR>(o, p.d_prev, lane, vo);
-    load_seg<E, kR>(go, p.d_prev, lane, vg);
-    load_seg<E, kR>(e, de, lane, ve);
-    load_seg<E, kR>(ge, de, lane, vge);
+    uint4 vo[kRo], vg[kRo], ve[kRe], vge[kRe];
+    load_seg<E, kRo>(o, p.d_prev, lane, vo);
+    load_seg<E, kRo>(go, p.d_prev, lane, vg);
+    load_seg<E, kRe>(e, de, lane, ve);
+    load_seg<E, kRe>(ge, de, lane, vge);
 #pragma unroll
-    for (int j = 0; j < kR; ++j) {
+    for (int j = 0; j < kRo; ++j) {
       float fo[N], fg[N];
       Vec<E>::unpack(vo[j], fo);
       Vec<E>::unpack(vg[j], fg);
@@ -219,7 +228,7 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock) junction_bwd_kernel(const 
     }
     oo = warp_sum(oo);
     dot = warp_sum(dot);
-    ee = warp_sum(sumsq_cached<E, kR>(ve));
+    ee = warp_sum(sumsq_cached<E, kRe>(ve));
     const float no = sqrtf(oo), ne = sqrtf(ee);
     const float s = no > 0.f ? ne / no : 0.f;
     const float co = no > 0.f ? dot / oo : 0.f;                    // (g_o . o) / ||o||^2
@@ -228,7 +237,7 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock) junction_bwd_kernel(const 
     keep_packed(vg);
     keep_packed(ve);
 #pragma unroll
-    for (int j = 0; j < kR; ++j) {
+    for (int j = 0; j < kRo; ++j) {
       const int k = (j * 32 + lane) * N;
       if (k < p.d_prev) {
         float fo[N], fg[N], r[N];
@@ -238,6 +247,10 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock) junction_bwd_kernel(const 
         for (int i = 0; i < N; ++i) r[i] = s * fmaf(-fo[i], co, fg[i]);
         st16(d_o + k, Vec<E>::pack(r));
       }
+    }
+#pragma unroll
+    for (int j = 0; j < kRe; ++j) {
+      const int k = (j * 32 + lane) * N;
       if (k < de) {
         float fe[N], fg[N], r[N];
         Vec<E>::unpack(ve[j], fe);
@@ -476,42 +489,53 @@ cudaError_t ring_launch(const JunctionParams& p, cudaStream_t s, bool& launched)
   return cudaGetLastError();
 }
 
-// Cached vectors per lane for a row whose segments are d_prev and d_next -
-// d_prev elements of `elt` bytes: the smallest of 1, 2, 4, 8 that holds both,
-// or 0 when a segment needs more.  At 12 vectors the backward needed 254
-// registers and ran ~10% slower than the TMA ring.
-int cache_vectors(int d_prev, int d_next, int elt) {
+// Cached vectors per lane for a segment of n elements of `elt` bytes: the
+// smallest of 1, 2, 4, 8 that holds it, or 0 when it needs more.  At 12 vectors
+// the backward needed 254 registers and ran ~10% slower than the TMA ring.
+int cache_vectors(int n, int elt) {
   const int per = 32 * (16 / elt);  // elements per cached vector across the warp
-  const int need_o = (d_prev + per - 1) / per, need_e = (d_next - d_prev + per - 1) / per;
-  const int need = need_o > need_e ? need_o : need_e;
   for (const int r : {1, 2, 4, 8})
-    if (need <= r) return r;
+    if (n <= r * per) return r;
   return 0;
 }
 
-template <typename E>
-cudaError_t fwd_launch(const JunctionParams& p, int r, unsigned blocks, cudaStream_t s) {
-  const dim3 b(32 * kRowsPerBlock);
-  switch (r) {
-    case 1: junction_fwd_kernel<E, 1><<<blocks, b, 0, s>>>(p); break;
-    case 2: junction_fwd_kernel<E, 2><<<blocks, b, 0, s>>>(p); break;
-    case 4: junction_fwd_kernel<E, 4><<<blocks, b, 0, s>>>(p); break;
-    case 8: junction_fwd_kernel<E, 8><<<blocks, b, 0, s>>>(p); break;
-    default: junction_fwd_kernel<E, 0><<<blocks, b, 0, s>>>(p); break;
-  }
-  return cudaGetLastError();
+// The kernel for segments of ro and re cached vectors per lane (streaming if
+// either does not fit).
+using JunctionKernel = void (*)(JunctionParams);
+
+template <typename E, bool kBwd, int kRo>
+JunctionKernel pick_re(int re) {
+#define MLS_PICK(R) \
+  if (re == R) return kBwd ? junction_bwd_kernel<E, kRo, R> : junction_fwd_kernel<E, kRo, R>;
+  MLS_PICK(1)
+  MLS_PICK(2)
+  MLS_PICK(4)
+#undef MLS_PICK
+  return kBwd ? junction_bwd_kernel<E, kRo, 8> : junction_fwd_kernel<E, kRo, 8>;
 }
 
-template <typename E>
-cudaError_t bwd_launch(const JunctionParams& p, int r, unsigned blocks, cudaStream_t s) {
-  const dim3 b(32 * kRowsPerBlock);
-  switch (r) {
-    case 1: junction_bwd_kernel<E, 1><<<blocks, b, 0, s>>>(p); break;
-    case 2: junction_bwd_kernel<E, 2><<<blocks, b, 0, s>>>(p); break;
-    case 4: junction_bwd_kernel<E, 4><<<blocks, b, 0, s>>>(p); break;
-    case 8: junction_bwd_kernel<E, 8><<<blocks, b, 0, s>>>(p); break;
-    default: junction_bwd_kernel<E, 0><<<blocks, b, 0, s>>>(p); break;
+template <typename E, bool kBwd>
+JunctionKernel pick_kernel(int ro, int re) {
+  if (ro == 0 || re == 0) return kBwd ? junction_bwd_kernel<E, 0, 0> : junction_fwd_kernel<E, 0, 0>;
+  switch (ro) {
+    case 1: return pick_re<E, kBwd, 1>(re);
+    case 2: return pick_re<E, kBwd, 2>(re);
+    case 4: return pick_re<E, kBwd, 4>(re);
+    default: return pick_re<E, kBwd, 8>(re);
   }
+}
+
+template <typename E, bool kBwd>
+cudaError_t junction_launch(const JunctionParams& p, cudaStream_t s) {
+  const long long blocks = (p.T + kRowsPerBlock - 1) / kRowsPerBlock;
+  if (blocks <= 0) return cudaSuccess;
+  const int ro = cache_vectors(p.d_prev, sizeof(E)), re = cache_vectors(p.d_next - p.d_prev, sizeof(E));
+  if (ro == 0 || re == 0) {
+    bool launched = false;
+    const cudaError_t e = ring_launch<E, kBwd>(p, s, launched);
+    if (e != cudaSuccess || launched) return e;
+  }
+  pick_kernel<E, kBwd>(ro, re)<<<static_cast<unsigned>(blocks), 32 * kRowsPerBlock, 0, s>>>(p);
   return cudaGetLastError();
 }
 
@@ -520,31 +544,11 @@ cudaError_t bwd_launch(const JunctionParams& p, int r, unsigned blocks, cudaStre
 // Register cache when a row fits 8 vectors per lane, else the TMA ring, else
 // (rows too wide for two ring buffers) the streaming kernel.
 cudaError_t launch_junction_fwd(const JunctionParams& p, bool fp32, cudaStream_t s) {
-  const long long blocks = (p.T + kRowsPerBlock - 1) / kRowsPerBlock;
-  if (blocks <= 0) return cudaSuccess;
-  const int r = cache_vectors(p.d_prev, p.d_next, fp32 ? 4 : 2);
-  if (r == 0) {
-    bool launched = false;
-    const cudaError_t e = fp32 ? ring_launch<float, false>(p, s, launched)
-                               : ring_launch<__nv_bfloat16, false>(p, s, launched);
-    if (e != cudaSuccess || launched) return e;
-  }
-  return fp32 ? fwd_launch<float>(p, r, static_cast<unsigned>(blocks), s)
-              : fwd_launch<__nv_bfloat16>(p, r, static_cast<unsigned>(blocks), s);
+  return fp32 ? junction_launch<float, false>(p, s) : junction_launch<__nv_bfloat16, false>(p, s);
 }
 
 cudaError_t launch_junction_bwd(const JunctionParams& p, bool fp32, cudaStream_t s) {
-  const long long blocks = (p.T + kRowsPerBlock - 1) / kRowsPerBlock;
-  if (blocks <= 0) return cudaSuccess;
-  const int r = cache_vectors(p.d_prev, p.d_next, fp32 ? 4 : 2);
-  if (r == 0) {
-    bool launched = false;
-    const cudaError_t e = fp32 ? ring_launch<float, true>(p, s, launched)
-                               : ring_launch<__nv_bfloat16, true>(p, s, launched);
-    if (e != cudaSuccess || launched) return e;
-  }
-  return fp32 ? bwd_launch<float>(p, r, static_cast<unsigned>(blocks), s)
-              : bwd_launch<__nv_bfloat16>(p, r, static_cast<unsigned>(blocks), s);
+  return fp32 ? junction_launch<float, true>(p, s) : junction_launch<__nv_bfloat16, true>(p, s);
 }
 
 cudaError_t setup_junction_kernels() {
