@@ -247,12 +247,12 @@ struct GemmCut {
 // about 0.33 us) and one per kSplitBytes written and read.  A split has to be
 // estimated kSplitGain faster, so that large launches stay whole.  Measured,
 // launch whole against split with its sum: 300 tokens, d = (96, 400), V = 30000
-// in fp32 (6 dH tiles of 938 k-blocks) 261 against 84 us; 100 tokens, d =
-// (512, 1024), V = 20000 (6 of 313) 117 against 87 us; 20000 tokens, d =
-// (512, 1024), V = 600 (dW, 18 of 313) 117 against 102 us; but 256 tokens, d =
-// (128, 256), V = 1024 in fp32 (2 of 32) 22 against 25 us.
+// in fp32 (6 dH tiles of 938 k-blocks) 261 against 73 us; 100 tokens, d =
+// (512, 1024), V = 20000 (6 of 313) 117 against 50 us; 20000 tokens, d =
+// (512, 1024), V = 600 (dW, 18 of 313) 117 against 78 us; 256 tokens, d = (128,
+// 256), V = 1024 in fp32 (2 of 32): a step of 55.9 against 53.1 us.
 constexpr int kSplitMinBlocks = 12, kSplitMost = 32;
-constexpr long long kSplitLaunch = 16, kSplitBytes = 1700000;
+constexpr long long kSplitLaunch = 8, kSplitBytes = 1700000;
 constexpr double kSplitGain = 0.95;
 // A launch estimated shorter than this (about 170 us) starts chained to its
 // predecessor, which saves some 3 us of launch latency.  A long one is launched
