@@ -80,23 +80,53 @@ struct UnitCoord {
   int ks;                // split of the reduction (0 unless GemmProblem::ksplit > 1)
 };
 
-// The j-th unit of this pair, or -1 when it has no more.
-__device__ __forceinline__ int pair_unit(const GemmParams& p, int pair, int npairs, int j) {
-  if (!p.two_class) {
-    const int t = pair + j * npairs;
-    return t < p.total_tiles ? t : -1;
+// The units of one pair, in order (see GemmParams).  Stepping costs an addition,
+// and decoding a unit's number two multiplications: the producer and the MMA
+// issuer are single threads, and a chain of divisions stood between one unit's
+// last k-block and the next one's first.  GEMM launch, divisions against this:
+// 100 tokens, d = (512, 1024), V = 20000 (units of 2 k-blocks) 42.9 -> 40.8 us;
+// 1531 tokens, d = (520, 1032, 2056), V = 32003 (24) 520 -> 514 us; unchanged
+// where units are long.
+struct PairUnits {
+  int u, step, left, stage;  // next unit, distance to the one after, units left of this stage
+  int prob;                  // problem of the last decoded unit (they only move up)
+  __device__ __forceinline__ void start(const GemmParams& p, int pair, int npairs) {
+    u = pair;
+    step = npairs;
+    prob = 0;
+    stage = p.two_class ? 0 : 2;
+    const int n = p.two_class ? p.n_long : p.total_tiles;
+    left = n > pair ? (n - pair + npairs - 1) / npairs : 0;
   }
-  const int r = p.n_long % npairs;
-  const int nl = p.n_long / npairs + (pair < r ? 1 : 0);
-  if (j < nl) return pair + j * npairs;
-  j -= nl;
-  const int n_short = p.total_tiles - p.n_long;
-  if (pair >= r) {
-    if (j < p.catchup) return p.n_long + (pair - r) + j * (npairs - r);
-    j -= p.catchup;
+  // The next unit of this pair, or -1 when it has no more.
+  __device__ __forceinline__ int next(const GemmParams& p, int pair, int npairs) {
+    while (left == 0) {
+      if (stage == 2) return -1;
+      const int r = p.n_long % npairs;
+      if (stage == 0 && pair >= r) {  // one long unit fewer: short units to catch up
+        u = p.n_long + (pair - r);
+        step = npairs - r;
+        left = p.catchup;
+        stage = 1;
+      } else {
+        const int first = p.n_long + p.catchup * (npairs - r) + pair;
+        u = first;
+        step = npairs;
+        left = p.total_tiles > first ? (p.total_tiles - first + npairs - 1) / npairs : 0;
+        stage = 2;
+      }
+    }
+    const int got = u;
+    u += step;
+    --left;
+    return got;
   }
-  const int s = p.catchup * (npairs - r) + pair + j * npairs;
-  return s < n_short ? p.n_long + s : -1;
+};
+
+// n / d by the multiplier and shift that the host made for d (FastDiv).
+__device__ __forceinline__ int fast_div(int n, const FastDiv& d) {
+  const unsigned t = __umulhi(d.mul, static_cast<unsigned>(n));
+  return static_cast<int>((t + ((static_cast<unsigned>(n) - t) >> d.s1)) >> d.s2);
 }
 
 // A is MN-major for this problem.
@@ -111,23 +141,22 @@ __device__ __forceinline__ bool wide_of(const GemmProblem& pr) {
   return kAMode == 2 && pr.wide != 0;
 }
 
+// `hint`: the problem of an earlier unit of this pair.
 template <int kAMode>
-__device__ __forceinline__ UnitCoord decode_unit(const GemmParams& p, int u) {
-  int i = 0;
+__device__ __forceinline__ UnitCoord decode_unit(const GemmParams& p, int u, int& hint) {
+  int i = hint;
   while (i + 1 < p.nprob && u >= p.prob[i + 1].tile_begin) ++i;
+  hint = i;
   const GemmProblem& pr = p.prob[i];
-  const int local = u - pr.tile_begin;
-  if (pr.m_fast) return {i, local % pr.tiles_m, local / pr.tiles_m, 1, 0};
-  if (wide_of<kAMode>(pr)) {
-    const int un = (pr.tiles_n + 1) >> 1;
-    const int tn = (local % un) * 2;
-    return {i, local / un, tn, pr.tiles_n - tn < 2 ? 1 : 2, 0};
-  }
+  int local = u - pr.tile_begin, ks = 0;
   if (kAMode == 2 && pr.ksplit > 1) {
-    const int tiles = pr.tiles_m * pr.tiles_n, t = local % tiles;
-    return {i, t / pr.tiles_n, t % pr.tiles_n, 1, local / tiles};
+    ks = fast_div(local, pr.div_tiles);
+    local -= ks * pr.tiles_m * pr.tiles_n;
   }
-  return {i, local / pr.tiles_n, local % pr.tiles_n, 1, 0};
+  const int q = fast_div(local, pr.div_inner), r = local - q * pr.inner;
+  if (pr.m_fast) return {i, r, q, 1, 0};
+  if (wide_of<kAMode>(pr)) return {i, q, 2 * r, pr.tiles_n - 2 * r < 2 ? 1 : 2, 0};
+  return {i, q, r, 1, ks};
 }
 
 // The k-blocks [begin, end) that a unit reduces.
@@ -159,8 +188,10 @@ __device__ __forceinline__ void gemm_producer(const GemmParams& p, uint32_t base
   int layout = -1;  // ring the stages were last filled in: 0 plain, 1 wide
   bool ok = true;
   int u;
-  for (int j = 0; ok && (u = pair_unit(p, pair, npairs, j)) >= 0; ++j) {
-    const UnitCoord uc = decode_unit<kAMode>(p, u);
+  PairUnits units;
+  units.start(p, pair, npairs);
+  while (ok && (u = units.next(p, pair, npairs)) >= 0) {
+    const UnitCoord uc = decode_unit<kAMode>(p, u, units.prob);
     const GemmProblem& pr = p.prob[uc.prob];
     MLS_CHECK(p.status, u < p.total_tiles && uc.prob < p.nprob && pr.a_map < kGemmMaxProblems &&
                             static_cast<long long>(uc.tm) * kPairM < pr.Mrows &&
@@ -265,8 +296,10 @@ __device__ __forceinline__ void gemm_mma(const GemmParams& p, uint32_t base, uin
   uint32_t phase = 0, wphase = 0, tiles = 0;
   bool ok = true;
   int u;
-  for (int j = 0; ok && (u = pair_unit(p, pair, npairs, j)) >= 0; ++j) {
-    const UnitCoord uc = decode_unit<kAMode>(p, u);
+  PairUnits units;
+  units.start(p, pair, npairs);
+  while (ok && (u = units.next(p, pair, npairs)) >= 0) {
+    const UnitCoord uc = decode_unit<kAMode>(p, u, units.prob);
     const GemmProblem& pr = p.prob[uc.prob];
     int kb_begin, kb_end;
     unit_kblocks<kTF32>(pr, uc, kb_begin, kb_end);
@@ -452,8 +485,10 @@ __device__ __forceinline__ void gemm_epilogue(const GemmParams& p, uint32_t base
   const uint32_t stage = base + GemmSmem::kStaging + static_cast<uint32_t>(warp) * 2 * GemmSmem::kChunk;
   bool aborted = false;
   int u;
-  for (int j = 0; !aborted && (u = pair_unit(p, pair, npairs, j)) >= 0; ++j) {
-    const UnitCoord uc = decode_unit<kAMode>(p, u);
+  PairUnits units;
+  units.start(p, pair, npairs);
+  while (!aborted && (u = units.next(p, pair, npairs)) >= 0) {
+    const UnitCoord uc = decode_unit<kAMode>(p, u, units.prob);
     const GemmProblem& pr = p.prob[uc.prob];
     for (int t = 0; t < uc.nt; ++t, ++tiles) {
       const uint32_t acc = tiles & 1u;
@@ -577,17 +612,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
 
 }  // namespace
 
+namespace {
+void number_units(GemmParams& p) {
+  for (int i = 0; i < p.nprob; ++i) {
+    GemmProblem& q = p.prob[i];
+    q.inner = q.m_fast ? q.tiles_m : q.wide ? (q.tiles_n + 1) / 2 : q.tiles_n;
+    q.div_inner = make_fast_div(q.inner);
+    q.div_tiles = make_fast_div(q.tiles_m * q.tiles_n);
+  }
+}
+}  // namespace
+
 // The verify step's first kernel.
-cudaError_t launch_gemm_stats(const GemmParams& p, bool tf32, int grid, cudaStream_t s) {
+cudaError_t launch_gemm_stats(GemmParams& p, bool tf32, int grid, cudaStream_t s) {
   if (p.total_tiles <= 0 || grid <= 0) return cudaSuccess;
+  number_units(p);
   if (tf32)
     gemm_kernel<true, 0, false, true><<<grid, kGemmThreads, kGemmSmem, s>>>(p);
   else
     gemm_kernel<false, 0, false, true><<<grid, kGemmThreads, kGemmSmem, s>>>(p);
   return cudaGetLastError();
 }
-cudaError_t launch_gemm_mixed(const GemmParams& p, bool tf32, int grid, cudaStream_t s) {
+cudaError_t launch_gemm_mixed(GemmParams& p, bool tf32, int grid, cudaStream_t s) {
   if (p.total_tiles <= 0 || grid <= 0) return cudaSuccess;
+  number_units(p);
   if (!p.chained) {
     if (tf32)
       gemm_kernel<true, 2, true, false><<<grid, kGemmThreads, kGemmSmem, s>>>(p);

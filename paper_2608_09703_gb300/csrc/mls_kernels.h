@@ -126,6 +126,20 @@ constexpr uint32_t kGemmBBytes = kGemmBHalf * 128;
 // inside the CTA's allocation.
 constexpr uint32_t kGemmSmem = kGemmStages * (kGemmABytes + kGemmBBytes) + 1024 + 1024 + 32768;
 
+// Division of n < 2^31 by d >= 1 as a multiplication (Granlund and Montgomery,
+// 1994): with l = ceil(log2 d), mul = floor(2^32 (2^l - d) / d) + 1, t the high
+// word of mul n, n / d = (t + ((n - t) >> min(l, 1))) >> max(l - 1, 0).
+struct FastDiv {
+  unsigned mul;
+  int s1, s2;
+};
+inline FastDiv make_fast_div(int d) {
+  int l = 0;
+  while ((1ll << l) < d) ++l;
+  return {static_cast<unsigned>(((1ull << 32) * ((1ull << l) - static_cast<unsigned>(d))) / static_cast<unsigned>(d) + 1),
+          l < 1 ? l : 1, l > 1 ? l - 1 : 0};
+}
+
 struct GemmProblem {
   int Mrows, Ncols, K;           // C is Mrows x Ncols, reduction length K
   int a_map, b_map;              // index into mapA / mapB
@@ -159,6 +173,10 @@ struct GemmProblem {
   // added afterwards (launch_split_sum).  Units are numbered split by split.
   int ksplit;                    // 0 or 1: one unit reduces all of K
   int kb_split;
+  // Unit numbering, filled by the launchers: `inner` consecutive units run along
+  // the fast dimension (tiles_m if m_fast, else the units of a tile row).
+  int inner;
+  FastDiv div_inner, div_tiles;  // by inner, and by tiles_m * tiles_n (split by split)
 };
 enum GemmEpilogue { kEpiPlain = 0, kEpiSoftmax = 1, kEpiArgmax = 2 };
 
@@ -360,9 +378,9 @@ constexpr int kEvalMergeTokens = 32;  // tokens per evaluation-merge block: one 
 cudaError_t launch_head_fwd(const HeadParams& p, bool tf32, bool tau_one, cudaStream_t s);
 cudaError_t launch_head_bwd(const HeadParams& p, bool tf32, bool tau_one, cudaStream_t s);
 // B MN-major, A's layout per problem (GemmProblem::a_mn): dW and dH in one launch.
-cudaError_t launch_gemm_mixed(const GemmParams& p, bool tf32, int grid, cudaStream_t s);
+cudaError_t launch_gemm_mixed(GemmParams& p, bool tf32, int grid, cudaStream_t s);
 // Both operands K-major, with the statistics epilogues (GemmProblem::epi).
-cudaError_t launch_gemm_stats(const GemmParams& p, bool tf32, int grid, cudaStream_t s);
+cudaError_t launch_gemm_stats(GemmParams& p, bool tf32, int grid, cudaStream_t s);
 cudaError_t launch_merge(const MergeParams& p, int blocks, cudaStream_t s);
 cudaError_t launch_final(const double* block_sum, const long long* block_cnt, int nblocks,
                          float* loss, cudaStream_t s);
