@@ -118,13 +118,15 @@ struct Plan {
   int band = 1;      // token tiles per band of the forward and evaluation launch order
   int band_bwd = 1;  // the same for the backward head kernel
   // forward
-  int S = 1, nparts = 0, merge_blocks = 0, eval_merge_blocks = 0;
+  TileSplit split = {};      // forward
+  int nparts = 0, merge_blocks = 0, eval_merge_blocks = 0;
   size_t off_part = 0, off_bsum = 0, off_bcnt = 0, fwd_bytes = 0;
   // backward
   long long group = 0, ngroups = 0;
   size_t off_invn = 0, off_G = 0, off_split = 0, bwd_bytes = 0;
   // pairwise evaluation
-  int eval_nvt = 0, eval_S = 1;
+  TileSplit eval_split = {};
+  int eval_nparts = 0;
   size_t off_epart = 0, off_eacc = 0, off_ecnt = 0, eval_bytes = 0;
   size_t total = 0;
 };
@@ -141,26 +143,6 @@ constexpr double kHeadCtaCost = 0.25;
 // vocabulary tiles): 33 splits (the head kernels' choice) 3.39 ms per call,
 // 7 splits 3.24 ms, which puts its per-pair cost near 1.2 tiles.
 constexpr double kEvalCtaCost = 1.25;
-int choose_splits(int ntt, long long tiles, int pairs, double cta_cost = kHeadCtaCost) {
-  if (ntt < 1) ntt = 1;
-  if (tiles < 1) return 1;
-  long long best = 1;
-  double best_cost = 1e300;
-  // of the S with the same tiles per pair, the smallest (fewest waves); trying every
-  // S cost a step of the 3-level suite some 10 us on the host
-  for (long long S = 1, per = tiles; S <= tiles && S <= 512;
-       S = per > 1 ? (tiles + per - 2) / (per - 1) : tiles + 1) {
-    per = (tiles + S - 1) / S;
-    const long long waves = (ntt * S + pairs - 1) / pairs;
-    const double cost = waves * (per + cta_cost);
-    if (cost < best_cost - 1e-9) {
-      best_cost = cost;
-      best = S;
-    }
-  }
-  return static_cast<int>(best);
-}
-
 // Token tiles per band of the head kernels' launch order (band_unit): the
 // pairs resident at one time re-read the hidden states of every sub-model for
 // the band's tokens once per vocabulary tile, so a band's H is kept within a
@@ -309,6 +291,67 @@ GemmCut cut_gemm(int M, const int32_t* d, long long T, long long gc, bool first,
   return c;
 }
 
+// Leaving some tiles to extra pairs (TileSplit) has to be estimated this much
+// faster.  Measured, all tiles in one wave of regular pairs against this: head
+// forward and backward of 1531 tokens, d = (520, 1032, 2056), V = 32003 (6 token
+// tiles x 12 splits of 10 or 11 tiles; 10 each and 12 runs of 3) 300 + 333 -> 285
+// + 318 us; evaluation of 2999 tokens, d = (1024, 3072), V = 49152 (12 x 6 of 32;
+// 31 each and 12 runs of 6) 765 -> 738 us.
+constexpr double kExtraGain = 0.985;
+TileSplit choose_splits(int ntt, long long tiles, int pairs, int band, double cta_cost = kHeadCtaCost) {
+  TileSplit sp = {};
+  sp.S = 1;
+  sp.band = band;
+  sp.ntt = ntt;
+  sp.main_end = sp.end = static_cast<int>(tiles);
+  if (ntt < 1) ntt = 1;
+  if (tiles < 1) return sp;
+  long long best = 1;
+  double best_cost = 1e300;
+  // of the S with the same tiles per pair, the smallest (fewest waves); trying every
+  // S cost a step of the 3-level suite some 10 us on the host
+  for (long long S = 1, per = tiles; S <= tiles && S <= 512;
+       S = per > 1 ? (tiles + per - 2) / (per - 1) : tiles + 1) {
+    per = (tiles + S - 1) / S;
+    const long long waves = (ntt * S + pairs - 1) / pairs;
+    const double cost = waves * (per + cta_cost);
+    if (cost < best_cost - 1e-9) {
+      best_cost = cost;
+      best = S;
+    }
+  }
+  sp.S = static_cast<int>(best);
+  if (band < ntt) return sp;  // several bands: pairs of one band share its hidden states in L2
+
+  // One wave of ntt x S pairs leaves `spare` pairs' SMs idle and, where S does not
+  // divide the tiles, makes some pairs take one tile more.  So the regular pairs
+  // may stop after `cap` tiles each, and the rest runs as short extra pairs on
+  // the spare SMs (TileSplit).
+  best_cost *= kExtraGain;
+  for (long long S = pairs / ntt; S >= 1 && S >= pairs / ntt - 1; --S) {
+    const long long spare = pairs - ntt * S;
+    if (spare < 1 || S > tiles) continue;
+    const long long most = (tiles - 1) / S;  // tiles per pair that leave some over
+    for (long long cap = most; cap >= 1 && cap >= most - 3; --cap) {
+      const long long left = tiles - S * cap;
+      for (long long E = 1; E <= 8 && E <= left; ++E) {
+        const long long run = (left + E - 1) / E;
+        if ((E - 1) * run >= left) continue;
+        const double rounds = static_cast<double>((ntt * E + spare - 1) / spare) * (run + cta_cost);
+        const double cost = cap + cta_cost > rounds ? cap + cta_cost : rounds;
+        if (cost < best_cost - 1e-9) {
+          best_cost = cost;
+          sp.S = static_cast<int>(S);
+          sp.main_end = static_cast<int>(S * cap);
+          sp.extra = static_cast<int>(E);
+          sp.run = static_cast<int>(run);
+        }
+      }
+    }
+  }
+  return sp;
+}
+
 int validate(const mls_problem* p) {
   if (!p || p->M < 1 || p->M > MLS_MAX_MODELS || p->T < 0 || p->V < 1 || p->V > INT_MAX ||
       p->T > INT_MAX || !p->d)
@@ -335,12 +378,12 @@ Plan make_plan(const mls_problem* p, int pairs, int gemm_pairs) {
   const long long T = p->T, V = p->V, M = p->M;
   pl.ntt = static_cast<int>(ceil_div(T, 2 * kHeadBM));  // token tiles of a CTA pair
   pl.nvt = static_cast<int>(ceil_div(V, kHeadBN));
-  pl.S = choose_splits(pl.ntt, pl.nvt, pairs);
-  pl.nparts = pl.S;
   long long sum_d = 0;
   for (int m = 0; m < p->M; ++m) sum_d += p->d[m];
   pl.band = choose_band(pl.ntt, 2LL * kHeadBM * sum_d * pl.elt, kBandBytesFwd);
   pl.band_bwd = choose_band(pl.ntt, 2LL * kHeadBM * sum_d * pl.elt, kBandBytesBwd);
+  pl.split = choose_splits(pl.ntt, pl.nvt, pairs, pl.band);
+  pl.nparts = pl.split.S + pl.split.extra;
   pl.merge_blocks = static_cast<int>(ceil_div(T, merge_tokens_per_block(pl.nparts)));
   pl.eval_merge_blocks = static_cast<int>(ceil_div(T, kEvalMergeTokens));
   size_t o = 0;
@@ -387,11 +430,11 @@ Plan make_plan(const mls_problem* p, int pairs, int gemm_pairs) {
   }
   pl.bwd_bytes = o;
 
-  pl.eval_nvt = static_cast<int>(ceil_div(V, eval_tile_cols(p->M)));
-  pl.eval_S = choose_splits(pl.ntt, pl.eval_nvt, pairs, kEvalCtaCost);
+  pl.eval_split = choose_splits(pl.ntt, ceil_div(V, eval_tile_cols(p->M)), pairs, pl.band, kEvalCtaCost);
+  pl.eval_nparts = pl.eval_split.S + pl.eval_split.extra;
   o = 0;
   pl.off_epart = o;
-  o = align_up(o + sizeof(float) * static_cast<size_t>(pl.eval_S) * kEvalFields * T);
+  o = align_up(o + sizeof(float) * static_cast<size_t>(pl.eval_nparts) * kEvalFields * T);
   pl.off_eacc = o;
   o = align_up(o + sizeof(double) * 2 * kMaxModels * kMaxModels * static_cast<size_t>(pl.eval_merge_blocks + 1));
   pl.off_ecnt = o;
@@ -450,7 +493,6 @@ void fill_head_common(HeadParams& hp, const mls_problem* p, const Plan& pl, cons
   for (int m = 0, j = 1; m < p->M; ++m)
     if (m != p->teacher) hp.order[j++] = m;
   for (int m = 0; m < p->M; ++m) hp.nk[m] = static_cast<int>(ceil_div(p->d[m], KE));
-  hp.ntt = pl.ntt;
   hp.T = p->T;
   hp.V = p->V;
   hp.L1 = 1.4426950408889634f;
@@ -554,10 +596,7 @@ extern "C" int mls_head_loss_fwd(const mls_problem* p, const void* const* H, con
   std::memset(&hp, 0, sizeof hp);
   fill_head_common(hp, p, pl, targets, dev->status);
   if ((rc = encode_head_maps(hp, p, pl, H, W))) return rc;
-  hp.vt_begin = 0;
-  hp.vt_end = pl.nvt;
-  hp.S = pl.S;
-  hp.band = pl.band;
+  hp.split = pl.split;
   hp.part = reinterpret_cast<float*>(wsb + pl.off_part);
   if ((rc = timed("head_fwd", s, [&] { return launch_head_fwd(hp, pl.elt == 4, p->tau == 1.0f, s); }))) return rc;
 
@@ -650,10 +689,11 @@ extern "C" int mls_head_loss_bwd(const mls_problem* p, const void* const* H, con
   for (long long g = 0; g < pl.ngroups; ++g) {
     const long long c0 = g * pl.group;
     const long long gc = (p->V - c0 < pl.group) ? p->V - c0 : pl.group;  // columns of this group
-    hp.vt_begin = static_cast<int>(g * tiles_per_group);
-    hp.vt_end = static_cast<int>(ceil_div(c0 + gc, kHeadBN));
-    hp.S = choose_splits(pl.ntt, hp.vt_end - hp.vt_begin, dev->head_pairs);
-    hp.band = pl.band_bwd;
+    const int vt0 = static_cast<int>(g * tiles_per_group);
+    hp.split = choose_splits(pl.ntt, ceil_div(c0 + gc, kHeadBN) - vt0, dev->head_pairs, pl.band_bwd);
+    hp.split.begin += vt0;
+    hp.split.main_end += vt0;
+    hp.split.end += vt0;
     hp.g_col0 = c0;
     if ((rc = timed("head_bwd", s, [&] { return launch_head_bwd(hp, tf32, p->tau == 1.0f, s); }))) return rc;
     // dW and dH of every sub-model in one persistent launch, the class with the
@@ -853,10 +893,7 @@ extern "C" int mls_head_loss_fwd_noalloc(const mls_problem* p, const void* const
   std::memset(&hp, 0, sizeof hp);
   fill_head_common(hp, p, pl, targets, dev->status);
   if ((rc = encode_head_maps(hp, p, pl, H, W))) return rc;
-  hp.vt_begin = 0;
-  hp.vt_end = pl.nvt;
-  hp.S = pl.S;
-  hp.band = pl.band;
+  hp.split = pl.split;
   hp.part = reinterpret_cast<float*>(wsb + pl.off_part);
   if ((rc = timed("head_fwd", s, [&] { return launch_head_fwd(hp, pl.elt == 4, p->tau == 1.0f, s); })))
     return rc;
@@ -934,10 +971,7 @@ extern "C" int mls_head_pairwise(const mls_problem* p, const void* const* H, con
     ep.order[2] = t;
   }
   for (int i = 0; i < p->M; ++i) ep.pos[ep.order[i]] = i;
-  ep.ntt = pl.ntt;
-  ep.nvt = pl.eval_nvt;
-  ep.S = pl.eval_S;
-  ep.band = pl.band;
+  ep.split = pl.eval_split;
   ep.T = p->T;
   ep.V = p->V;
   ep.L1 = 1.4426950408889634f;
@@ -948,7 +982,7 @@ extern "C" int mls_head_pairwise(const mls_problem* p, const void* const* H, con
   EvalMergeParams mp;
   std::memset(&mp, 0, sizeof mp);
   mp.part = ep.part;
-  mp.nparts = ep.S;
+  mp.nparts = pl.eval_nparts;
   mp.M = p->M;
   mp.T = p->T;
   mp.V = p->V;

@@ -78,13 +78,13 @@ __host__ __device__ constexpr int dfield(int s, int j) { return kD + s * 3 + (j 
 
 template <bool kTF32, int kM>
 __device__ __forceinline__ void eval_producer(const EvalParams& p, uint32_t base, int row0,
-                                              uint32_t rank, int split, volatile int* abort_flag) {
+                                              uint32_t rank, const PairTiles& pt, volatile int* abort_flag) {
   using Sm = EvalSmem<kM>;
   constexpr int KE = kTF32 ? 32 : 64;
   int stage = 0;
   uint32_t phase = 0, filled = 0, lastpar = 0;
   bool ok = true;
-  for (int vt = split; ok && vt < p.nvt; vt += p.S) {
+  for (int vt = pt.first; ok && vt < pt.end; vt += pt.stride) {
     for (int i = 0; ok && i < kM; ++i) {
       const int m = p.order[i];
       for (int kb = 0; kb < p.nk[m]; ++kb) {
@@ -121,14 +121,14 @@ __device__ __forceinline__ void eval_producer(const EvalParams& p, uint32_t base
 // of q = 0 (free0); the others wait for it to have finished tile j - 1 (free1).
 template <bool kTF32, int kM>
 __device__ __forceinline__ void eval_mma(const EvalParams& p, uint32_t base, uint32_t tmem,
-                                         int split, volatile int* abort_flag) {
+                                         const PairTiles& pt, volatile int* abort_flag) {
   using Sm = EvalSmem<kM>;
   constexpr uint32_t kIdesc = make_idesc(2 * kHeadBM, Sm::kN, kTF32, false, false);
   int stage = 0;
   uint32_t phase = 0;
   bool ok = true;
   int j = 0;
-  for (int vt = split; ok && vt < p.nvt; vt += p.S, ++j) {
+  for (int vt = pt.first; ok && vt < pt.end; vt += pt.stride, ++j) {
     for (int i = 0; ok && i < kM; ++i) {
       const int m = p.order[i];
       if (j > 0 && i <= 1 &&
@@ -174,14 +174,14 @@ __device__ __forceinline__ void eval_mma(const EvalParams& p, uint32_t base, uin
 // and the pass over units 0 and 1 under unit 2's MMAs.
 template <bool kTF32>
 __device__ __forceinline__ void eval_mma_slots(const EvalParams& p, uint32_t base, uint32_t tmem,
-                                               int split, volatile int* abort_flag) {
+                                               const PairTiles& pt, volatile int* abort_flag) {
   using Sm = EvalSmem<3>;
   constexpr uint32_t kIdesc = make_idesc(2 * kHeadBM, Sm::kN, kTF32, false, false);
   int stage = 0;
   uint32_t phase = 0;
   bool ok = true;
   int j = 0;
-  for (int vt = split; ok && vt < p.nvt; vt += p.S, ++j) {
+  for (int vt = pt.first; ok && vt < pt.end; vt += pt.stride, ++j) {
     const uint32_t sa = static_cast<uint32_t>(j & 1) * Sm::kN, sb = Sm::kN - sa;
     for (int i = 0; ok && i < 3; ++i) {
       const int m = p.order[i];
@@ -419,7 +419,7 @@ __device__ __forceinline__ void fold_pair(EvalState<3>& st, int a, int b, const 
 // Every pass runs with its units' maxima already folded in, so its chunks are
 // independent of one another.
 __device__ __forceinline__ bool eval_slots_main(const EvalParams& p, uint32_t base, uint32_t tl,
-                                                int split, int half, int lane,
+                                                const PairTiles& pt, int half, int lane,
                                                 volatile int* abort_flag, EvalState<3>& st) {
   using Sm = EvalSmem<3>;
   constexpr int kHalf = Sm::kN / 2;  // 128 columns per thread
@@ -427,7 +427,7 @@ __device__ __forceinline__ bool eval_slots_main(const EvalParams& p, uint32_t ba
   const float L1 = p.L1;
   const long long V = p.V;
   int j = 0;
-  for (int vt = split; vt < p.nvt; vt += p.S, ++j) {
+  for (int vt = pt.first; vt < pt.end; vt += pt.stride, ++j) {
     const uint32_t par = static_cast<uint32_t>(j) & 1u;
     const uint32_t sa = par * Sm::kN, sb = Sm::kN - sa;
     const long long tcol = static_cast<long long>(vt) * Sm::kN + half * kHalf;
@@ -527,7 +527,7 @@ __device__ __forceinline__ bool eval_slots_main(const EvalParams& p, uint32_t ba
 
 template <int kM>
 __device__ __forceinline__ void eval_epilogue(const EvalParams& p, uint32_t base, uint32_t tmem,
-                                              float* xchg, int row_base, int split, int warp,
+                                              float* xchg, int row_base, const PairTiles& pt, int warp,
                                               int lane, volatile int* abort_flag) {
   using Sm = EvalSmem<kM>;
   constexpr int kHalf = Sm::kN / 2;  // columns per thread
@@ -547,10 +547,10 @@ __device__ __forceinline__ void eval_epilogue(const EvalParams& p, uint32_t base
     for (int j = 0; j < kM; ++j) st.d[q][j] = 0.f;
   }
   if constexpr (eval_slotted(kM)) {
-    eval_slots_main(p, base, tl, split, half, lane, abort_flag, st);
+    eval_slots_main(p, base, tl, pt, half, lane, abort_flag, st);
   } else {
   int j = 0;
-  for (int vt = split; vt < p.nvt; vt += p.S, ++j) {
+  for (int vt = pt.first; vt < pt.end; vt += pt.stride, ++j) {
     const bool ok = mbar_wait(Sm::accf(base, j), static_cast<uint32_t>(j >> 1) & 1u, abort_flag, p.status);
     if (!__all_sync(0xffffffffu, ok)) break;
     tc_fence_after();
@@ -595,7 +595,7 @@ __device__ __forceinline__ void eval_epilogue(const EvalParams& p, uint32_t base
   }
   named_bar_sync(1, kHeadEpiWarps * 32);
   if (half == 1 || row >= p.T) return;
-  float* P = p.part + static_cast<long long>(split) * kEvalFields * p.T + row;
+  float* P = p.part + static_cast<long long>(pt.split) * kEvalFields * p.T + row;
 #pragma unroll
   for (int q = 0; q < kM; ++q) {
     const int s = p.order[q];
@@ -626,9 +626,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kHeadThreads, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + Sm::kTmemSlot);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
-  int tt, split;
-  band_unit(static_cast<int>(blockIdx.x >> 1), p.ntt, p.S, p.band, tt, split);
-  const int row_base = tt * 2 * kHeadBM + static_cast<int>(rank) * kHeadBM;
+  const PairTiles pt = p.split.tiles_of(static_cast<int>(blockIdx.x >> 1));
+  const int row_base = pt.tt * 2 * kHeadBM + static_cast<int>(rank) * kHeadBM;
 
   if (threadIdx.x == 0) {
     *abort_flag = 0;
@@ -668,21 +667,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kHeadThreads, 1)
     regs_decrease<kHeadCtlRegs>();
     if (warp == kHeadEpiWarps) {
       if (lane == 0) {
-        eval_producer<kTF32, kM>(p, base, row_base, rank, split, abort_flag);
+        eval_producer<kTF32, kM>(p, base, row_base, rank, pt, abort_flag);
         chain_trigger();
       }
     } else if (warp == kHeadEpiWarps + 1) {
       if (lane == 0 && rank == 0) {
         if constexpr (eval_slotted(kM))
-          eval_mma_slots<kTF32>(p, base, tmem, split, abort_flag);
+          eval_mma_slots<kTF32>(p, base, tmem, pt, abort_flag);
         else
-          eval_mma<kTF32, kM>(p, base, tmem, split, abort_flag);
+          eval_mma<kTF32, kM>(p, base, tmem, pt, abort_flag);
       }
       __syncwarp();
     }
   } else {
     regs_increase<kHeadEpiRegs>();
-    eval_epilogue<kM>(p, base, tmem, reinterpret_cast<float*>(gbase + Sm::kX), row_base, split,
+    eval_epilogue<kM>(p, base, tmem, reinterpret_cast<float*>(gbase + Sm::kX), row_base, pt,
                       warp, lane, abort_flag);
   }
 
@@ -852,7 +851,7 @@ cudaError_t launch_eval_m(const EvalParams& p, bool tf32, int grid, cudaStream_t
 }
 
 cudaError_t launch_eval(const EvalParams& p, bool tf32, cudaStream_t s) {
-  const int grid = 2 * p.ntt * p.S;
+  const int grid = 2 * p.split.pairs();
   if (grid <= 0) return cudaSuccess;
   switch (p.M) {
     case 1: return launch_eval_m<1>(p, tf32, grid, s);

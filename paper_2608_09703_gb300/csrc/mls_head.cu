@@ -61,7 +61,8 @@ struct HeadSmem {
   }
   static constexpr uint32_t kTmemSlot = kBar + 8u * (2 * kHeadStages + 5);
   static constexpr uint32_t kAbort = kTmemSlot + 4;
-  static constexpr uint32_t kEnd = kAbort + 4;
+  static constexpr uint32_t kTiles = kAbort + 4;  // this pair's tiles: first, end, stride, split
+  static constexpr uint32_t kEnd = kTiles + 16;
 };
 static_assert(HeadSmem::kEnd + 1024 <= kHeadSmem, "head shared memory map overflows");
 static_assert(kPartFields * kMaxModels * kHeadBM * 4 <= kHeadStaging,
@@ -73,7 +74,7 @@ constexpr uint64_t kDrainNs = 100000000ull;     // bound for shutdown waits
 // ------------------------------------------------------------------ producer
 template <bool kTF32>
 __device__ __forceinline__ void head_producer(const HeadParams& p, uint32_t base, int row0,
-                                              uint32_t rank, int split, volatile int* abort_flag) {
+                                              uint32_t rank, const volatile int* tiles, volatile int* abort_flag) {
   constexpr int KE = kTF32 ? 32 : 64;  // elements in 128 bytes of K
   int stage = 0;
   uint32_t phase = 0, filled = 0, lastpar = 0;
@@ -81,10 +82,10 @@ __device__ __forceinline__ void head_producer(const HeadParams& p, uint32_t base
   // Test hook (off unless the host sets it): the first pair issues nothing for
   // its first stage, so the MMA issuer's wait on that stage must run out.
   bool stall = p.test_stall && (blockIdx.x >> 1) == 0;
-  for (int vt = p.vt_begin + split; ok && vt < p.vt_end; vt += p.S) {
+  for (int vt = tiles[0]; ok && vt < tiles[1]; vt += tiles[2]) {
     for (int u = 0; ok && u < p.M; ++u) {
       const int m = p.order[u];
-      MLS_CHECK(p.status, m >= 0 && m < p.M && split < p.S &&
+      MLS_CHECK(p.status, m >= 0 && m < p.M && tiles[3] < p.split.S + p.split.extra &&
                               static_cast<long long>(vt) * kHeadBN < p.V + kHeadBN);
       for (int kb = 0; kb < p.nk[m]; ++kb) {
         if (!mbar_wait(HeadSmem::empty(base, stage), phase ^ 1u, abort_flag, p.status)) {
@@ -130,13 +131,13 @@ __device__ __forceinline__ void head_producer(const HeadParams& p, uint32_t base
 // ------------------------------------------------------------------ MMA issuer
 template <bool kTF32>
 __device__ __forceinline__ void head_mma(const HeadParams& p, uint32_t base, uint32_t tmem,
-                                         int split, volatile int* abort_flag) {
+                                         const volatile int* tiles, volatile int* abort_flag) {
   constexpr uint32_t kIdesc = make_idesc(2 * kHeadBM, kHeadBN, kTF32, false, false);
   constexpr uint16_t kBoth = 0x3;
   int stage = 0;
   uint32_t phase = 0, acc = 0, acc_par = 0;
   bool ok = true;
-  for (int vt = p.vt_begin + split; ok && vt < p.vt_end; vt += p.S) {
+  for (int vt = tiles[0]; ok && vt < tiles[1]; vt += tiles[2]) {
     for (int u = 0; ok && u < p.M; ++u) {
       const int m = p.order[u];
       if (!mbar_wait(HeadSmem::acce(base, acc), acc_par ^ 1u, abort_flag, p.status)) {
@@ -329,7 +330,7 @@ __device__ __forceinline__ int merged_argmax(float ma, int aa, float mb, int ab)
 
 template <bool kTauOne>
 __device__ __forceinline__ void fwd_epilogue(const HeadParams& p, uint32_t base, uint32_t tmem,
-                                             float* xchg, int row_base, int split, int warp,
+                                             float* xchg, int row_base, const volatile int* tiles, int warp,
                                              int lane, volatile int* abort_flag) {
   const int quad = warp & 3, half = warp >> 2;
   const long long row = static_cast<long long>(row_base) + quad * 32 + lane;
@@ -353,7 +354,7 @@ __device__ __forceinline__ void fwd_epilogue(const HeadParams& p, uint32_t base,
   uint32_t acc = 0, acc_par = 0;
 
   bool aborted = false;
-  for (int vt = p.vt_begin + split; !aborted && vt < p.vt_end; vt += p.S) {
+  for (int vt = tiles[0]; !aborted && vt < tiles[1]; vt += tiles[2]) {
     const long long col0 = static_cast<long long>(vt) * kHeadBN + half * 128;
     const int nvalid = static_cast<int>(max(0LL, min(128LL, p.V - col0)));
     const int yl = y >= 0 ? static_cast<int>(y - col0) : -1;
@@ -422,8 +423,8 @@ __device__ __forceinline__ void fwd_epilogue(const HeadParams& p, uint32_t base,
   const float accT = (mT == -INFINITY ? 0.f : fat * (aT + (mT - mTm) * Lt * stT)) +
                      (mT1 == -INFINITY ? 0.f : fbt * (X(kPartAcc, 0) + (mT1 - mTm) * Lt * stT1));
   const long long MT = static_cast<long long>(p.M) * p.T;
-  MLS_CHECK(p.status, split < p.S && row < p.T);
-  float* P = p.part + static_cast<long long>(split) * kPartFields * MT;
+  MLS_CHECK(p.status, tiles[3] < p.split.S + p.split.extra && row < p.T);
+  float* P = p.part + static_cast<long long>(tiles[3]) * kPartFields * MT;
   {
     float* Pt = P + static_cast<long long>(p.order[0]) * p.T + row;
     Pt[kPartMax * MT] = mTm;
@@ -571,7 +572,7 @@ __device__ __forceinline__ void bwd_student(uint32_t ta, int nvalid, int yl, flo
 
 template <bool kTauOne, bool kTF32>
 __device__ __forceinline__ void bwd_epilogue(const HeadParams& p, uint32_t base, uint32_t tmem,
-                                             int row_base, int split, int warp, int lane,
+                                             int row_base, const volatile int* tiles, int warp, int lane,
                                              volatile int* abort_flag) {
   const int quad = warp & 3, half = warp >> 2;
   const long long row = static_cast<long long>(row_base) + quad * 32 + lane;
@@ -610,7 +611,7 @@ __device__ __forceinline__ void bwd_epilogue(const HeadParams& p, uint32_t base,
   float q[128];
   uint32_t acc = 0, acc_par = 0;
 
-  for (int vt = p.vt_begin + split; vt < p.vt_end; vt += p.S) {
+  for (int vt = tiles[0]; vt < tiles[1]; vt += tiles[2]) {
     const long long col0 = static_cast<long long>(vt) * kHeadBN + half * 128;
     const int nvalid = static_cast<int>(max(0LL, min(128LL, p.V - col0)));
     const int yl = y >= 0 ? static_cast<int>(y - col0) : -1;
@@ -665,9 +666,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kHeadThreads, 1)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
-  int tt, split;
-  band_unit(static_cast<int>(blockIdx.x >> 1), p.ntt, p.S, p.band, tt, split);
-  const int row_base = tt * 2 * kHeadBM + static_cast<int>(rank) * kHeadBM;  // this CTA's tokens
+  // The bounds of the tile loops are read from shared memory at every tile: in
+  // registers they cost the epilogue, which is out of them, 8% of the forward.
+  volatile int* tiles = reinterpret_cast<volatile int*>(gbase + HeadSmem::kTiles);
+  int row_base;  // this CTA's tokens
+  {
+    const PairTiles pt = p.split.tiles_of(static_cast<int>(blockIdx.x >> 1));
+    row_base = pt.tt * 2 * kHeadBM + static_cast<int>(rank) * kHeadBM;
+    if (threadIdx.x == 0) {
+      tiles[0] = pt.first;
+      tiles[1] = pt.end;
+      tiles[2] = pt.stride;
+      tiles[3] = pt.split;
+    }
+  }
 
   if (threadIdx.x == 0) {
     *abort_flag = 0;
@@ -701,20 +713,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kHeadThreads, 1)
     regs_decrease<kHeadCtlRegs>();
     if (warp == kHeadEpiWarps) {
       if (lane == 0) {
-        head_producer<kTF32>(p, base, row_base, rank, split, abort_flag);
+        head_producer<kTF32>(p, base, row_base, rank, tiles, abort_flag);
         chain_trigger();
       }
     } else if (warp == kHeadEpiWarps + 1) {
-      if (lane == 0 && rank == 0) head_mma<kTF32>(p, base, tmem, split, abort_flag);
+      if (lane == 0 && rank == 0) head_mma<kTF32>(p, base, tmem, tiles, abort_flag);
       __syncwarp();
     }
   } else {
     regs_increase<kHeadEpiRegs>();
     if constexpr (kMode == kModeFwd)
       fwd_epilogue<kTauOne>(p, base, tmem, reinterpret_cast<float*>(gbase + HeadSmem::kStage),
-                            row_base, split, warp, lane, abort_flag);
+                            row_base, tiles, warp, lane, abort_flag);
     else
-      bwd_epilogue<kTauOne, kTF32>(p, base, tmem, row_base, split, warp, lane, abort_flag);
+      bwd_epilogue<kTauOne, kTF32>(p, base, tmem, row_base, tiles, warp, lane, abort_flag);
   }
 
   tc_fence_before();
@@ -736,7 +748,7 @@ cudaError_t launch_mode(const HeadParams& p, int grid, cudaStream_t s) {
 
 template <int kMode>
 cudaError_t launch_head(const HeadParams& p, bool tf32, bool tau_one, cudaStream_t s) {
-  const int grid = 2 * p.ntt * p.S;  // CTA pairs
+  const int grid = 2 * p.split.pairs();
   if (grid <= 0) return cudaSuccess;
   if (tf32) return tau_one ? launch_mode<kMode, true, true>(p, grid, s) : launch_mode<kMode, true, false>(p, grid, s);
   return tau_one ? launch_mode<kMode, false, true>(p, grid, s) : launch_mode<kMode, false, false>(p, grid, s);

@@ -75,6 +75,38 @@ __host__ __device__ inline void band_unit(int pair, int ntt, int S, int band, in
   split = i / nb;
 }
 
+// The vocabulary tiles of one pair: vt = first, first + stride, ... < end, and the
+// partial-state slot `split` of its token tile tt.  Regular pairs (ntt x S) share
+// the tiles [begin, main_end) of every token tile; what is left of it is cut into
+// `extra` runs of `run` tiles per token tile, which further pairs take on the SMs
+// that the regular ones leave free (main_end == end: none).
+struct PairTiles {
+  int tt, split, first, end, stride;
+};
+struct TileSplit {
+  int ntt, S, band;              // token tiles, regular pairs per token tile, band_unit's band
+  int begin, main_end, end;      // vocabulary tiles
+  int extra, run;
+  __host__ __device__ int pairs() const { return ntt * (S + extra); }
+  __host__ __device__ inline PairTiles tiles_of(int pair) const {
+    PairTiles t;
+    if (pair < ntt * S) {
+      band_unit(pair, ntt, S, band, t.tt, t.split);
+      t.first = begin + t.split;
+      t.end = main_end;
+      t.stride = S;
+    } else {
+      const int e = pair - ntt * S, piece = e / ntt;
+      t.tt = e - piece * ntt;
+      t.split = S + piece;
+      t.first = main_end + piece * run;
+      t.end = t.first + run < end ? t.first + run : end;
+      t.stride = 1;
+    }
+    return t;
+  }
+};
+
 // Partial row state written by the forward head kernel, per (partial, field, model, token).
 // kPartAcc holds, for a student, sum_v q~_v z_m[v] with q~ relative to the
 // teacher's running maximum of the same partial; for the teacher,
@@ -87,10 +119,7 @@ struct HeadParams {
   int M;
   int order[kMaxModels];         // order[0] = teacher, then the students
   int nk[kMaxModels];            // k-blocks (128 bytes of K each) of model m
-  int ntt;                       // token tiles of 2 * kHeadBM (one per CTA pair)
-  int vt_begin, vt_end;          // vocabulary tiles handled by this launch
-  int S;                         // CTAs per token tile (vocabulary splits)
-  int band;                      // token tiles per band of the launch order (band_unit)
+  TileSplit split;               // token tiles of 2 * kHeadBM, vocabulary tiles of kHeadBN
   long long T, V;
   float L1;                      // log2(e)
   float Ltau;                    // log2(e) / tau
@@ -98,7 +127,7 @@ struct HeadParams {
   int* status;
   int test_stall;                // test hook: see head_producer (0 in normal use)
   // forward
-  float* part;                   // [S][kPartFields][M][T]
+  float* part;                   // [S + extra][kPartFields][M][T]
   // backward
   const float* stats;            // [2][M][T]: logsumexp(z), logsumexp(z/tau)
   const float* inv_n;            // device scalar 1/N (0 if N == 0)
@@ -244,14 +273,11 @@ struct EvalParams {
                                  // widest, narrowest, middle)
   int pos[kMaxModels];           // pos[order[i]] = i
   int nk[kMaxModels];
-  int ntt;                       // token tiles of 256 (one per CTA pair)
-  int nvt;                       // vocabulary tiles of eval_tile_cols(M) columns
-  int S;                         // CTA pairs per token tile
-  int band;                      // token tiles per band of the launch order (band_unit)
+  TileSplit split;               // token tiles of 256, vocabulary tiles of eval_tile_cols(M)
   long long T, V;
   float L1;
   int* status;
-  float* part;                   // [S][kEvalFields][T]
+  float* part;                   // [S + extra][kEvalFields][T]
 };
 
 struct EvalMergeParams {
