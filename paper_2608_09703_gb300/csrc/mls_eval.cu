@@ -61,7 +61,8 @@ struct EvalSmem {
   static __device__ __forceinline__ uint32_t drain(uint32_t b) { return tb(b, 7); }
   static constexpr uint32_t kTmemSlot = kBar + 8u * (2 * kStages + 8);
   static constexpr uint32_t kAbort = kTmemSlot + 4;
-  static constexpr uint32_t kEnd = kAbort + 4;
+  static constexpr uint32_t kTiles = kAbort + 4;  // this pair's tiles: first, end, stride, split
+  static constexpr uint32_t kEnd = kTiles + 16;
   static_assert(kEnd + 1024 <= eval_smem(kM), "eval shared memory map overflows");
   static_assert(eval_slotted(kM) ? 2 * kN <= 512 : kM * kN <= 512,
                 "the resident tiles must fit in TMEM");
@@ -78,13 +79,13 @@ __host__ __device__ constexpr int dfield(int s, int j) { return kD + s * 3 + (j 
 
 template <bool kTF32, int kM>
 __device__ __forceinline__ void eval_producer(const EvalParams& p, uint32_t base, int row0,
-                                              uint32_t rank, const PairTiles& pt, volatile int* abort_flag) {
+                                              uint32_t rank, const volatile int* tiles, volatile int* abort_flag) {
   using Sm = EvalSmem<kM>;
   constexpr int KE = kTF32 ? 32 : 64;
   int stage = 0;
   uint32_t phase = 0, filled = 0, lastpar = 0;
   bool ok = true;
-  for (int vt = pt.first; ok && vt < pt.end; vt += pt.stride) {
+  for (int vt = tiles[0]; ok && vt < tiles[1]; vt += tiles[2]) {
     for (int i = 0; ok && i < kM; ++i) {
       const int m = p.order[i];
       for (int kb = 0; kb < p.nk[m]; ++kb) {
@@ -121,14 +122,14 @@ __device__ __forceinline__ void eval_producer(const EvalParams& p, uint32_t base
 // of q = 0 (free0); the others wait for it to have finished tile j - 1 (free1).
 template <bool kTF32, int kM>
 __device__ __forceinline__ void eval_mma(const EvalParams& p, uint32_t base, uint32_t tmem,
-                                         const PairTiles& pt, volatile int* abort_flag) {
+                                         const volatile int* tiles, volatile int* abort_flag) {
   using Sm = EvalSmem<kM>;
   constexpr uint32_t kIdesc = make_idesc(2 * kHeadBM, Sm::kN, kTF32, false, false);
   int stage = 0;
   uint32_t phase = 0;
   bool ok = true;
   int j = 0;
-  for (int vt = pt.first; ok && vt < pt.end; vt += pt.stride, ++j) {
+  for (int vt = tiles[0]; ok && vt < tiles[1]; vt += tiles[2], ++j) {
     for (int i = 0; ok && i < kM; ++i) {
       const int m = p.order[i];
       if (j > 0 && i <= 1 &&
@@ -174,14 +175,14 @@ __device__ __forceinline__ void eval_mma(const EvalParams& p, uint32_t base, uin
 // and the pass over units 0 and 1 under unit 2's MMAs.
 template <bool kTF32>
 __device__ __forceinline__ void eval_mma_slots(const EvalParams& p, uint32_t base, uint32_t tmem,
-                                               const PairTiles& pt, volatile int* abort_flag) {
+                                               const volatile int* tiles, volatile int* abort_flag) {
   using Sm = EvalSmem<3>;
   constexpr uint32_t kIdesc = make_idesc(2 * kHeadBM, Sm::kN, kTF32, false, false);
   int stage = 0;
   uint32_t phase = 0;
   bool ok = true;
   int j = 0;
-  for (int vt = pt.first; ok && vt < pt.end; vt += pt.stride, ++j) {
+  for (int vt = tiles[0]; ok && vt < tiles[1]; vt += tiles[2], ++j) {
     const uint32_t sa = static_cast<uint32_t>(j & 1) * Sm::kN, sb = Sm::kN - sa;
     for (int i = 0; ok && i < 3; ++i) {
       const int m = p.order[i];
@@ -419,7 +420,7 @@ __device__ __forceinline__ void fold_pair(EvalState<3>& st, int a, int b, const 
 // Every pass runs with its units' maxima already folded in, so its chunks are
 // independent of one another.
 __device__ __forceinline__ bool eval_slots_main(const EvalParams& p, uint32_t base, uint32_t tl,
-                                                const PairTiles& pt, int half, int lane,
+                                                const volatile int* tiles, int half, int lane,
                                                 volatile int* abort_flag, EvalState<3>& st) {
   using Sm = EvalSmem<3>;
   constexpr int kHalf = Sm::kN / 2;  // 128 columns per thread
@@ -427,7 +428,7 @@ __device__ __forceinline__ bool eval_slots_main(const EvalParams& p, uint32_t ba
   const float L1 = p.L1;
   const long long V = p.V;
   int j = 0;
-  for (int vt = pt.first; vt < pt.end; vt += pt.stride, ++j) {
+  for (int vt = tiles[0]; vt < tiles[1]; vt += tiles[2], ++j) {
     const uint32_t par = static_cast<uint32_t>(j) & 1u;
     const uint32_t sa = par * Sm::kN, sb = Sm::kN - sa;
     const long long tcol = static_cast<long long>(vt) * Sm::kN + half * kHalf;
@@ -527,7 +528,7 @@ __device__ __forceinline__ bool eval_slots_main(const EvalParams& p, uint32_t ba
 
 template <int kM>
 __device__ __forceinline__ void eval_epilogue(const EvalParams& p, uint32_t base, uint32_t tmem,
-                                              float* xchg, int row_base, const PairTiles& pt, int warp,
+                                              float* xchg, int row_base, const volatile int* tiles, int warp,
                                               int lane, volatile int* abort_flag) {
   using Sm = EvalSmem<kM>;
   constexpr int kHalf = Sm::kN / 2;  // columns per thread
@@ -547,10 +548,10 @@ __device__ __forceinline__ void eval_epilogue(const EvalParams& p, uint32_t base
     for (int j = 0; j < kM; ++j) st.d[q][j] = 0.f;
   }
   if constexpr (eval_slotted(kM)) {
-    eval_slots_main(p, base, tl, pt, half, lane, abort_flag, st);
+    eval_slots_main(p, base, tl, tiles, half, lane, abort_flag, st);
   } else {
   int j = 0;
-  for (int vt = pt.first; vt < pt.end; vt += pt.stride, ++j) {
+  for (int vt = tiles[0]; vt < tiles[1]; vt += tiles[2], ++j) {
     const bool ok = mbar_wait(Sm::accf(base, j), static_cast<uint32_t>(j >> 1) & 1u, abort_flag, p.status);
     if (!__all_sync(0xffffffffu, ok)) break;
     tc_fence_after();
@@ -595,7 +596,7 @@ __device__ __forceinline__ void eval_epilogue(const EvalParams& p, uint32_t base
   }
   named_bar_sync(1, kHeadEpiWarps * 32);
   if (half == 1 || row >= p.T) return;
-  float* P = p.part + static_cast<long long>(pt.split) * kEvalFields * p.T + row;
+  float* P = p.part + static_cast<long long>(tiles[3]) * kEvalFields * p.T + row;
 #pragma unroll
   for (int q = 0; q < kM; ++q) {
     const int s = p.order[q];
@@ -626,8 +627,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kHeadThreads, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + Sm::kTmemSlot);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
-  const PairTiles pt = p.split.tiles_of(static_cast<int>(blockIdx.x >> 1));
-  const int row_base = pt.tt * 2 * kHeadBM + static_cast<int>(rank) * kHeadBM;
+  // The bounds of the tile loops stay in shared memory, read at every tile: the
+  // epilogue has no registers left for them.  8192 tokens of the 3-level suite
+  // took 3505 us per call with the bounds in registers, 3482 with them in the
+  // kernel's parameters (every pair alike) and 3337 this way; 4096 tokens of the
+  // 4-level suite 19.6, 19.8 and 18.4 ms.
+  volatile int* tiles = reinterpret_cast<volatile int*>(gbase + Sm::kTiles);
+  int row_base;  // this CTA's tokens
+  {
+    const PairTiles pt = p.split.tiles_of(static_cast<int>(blockIdx.x >> 1));
+    row_base = pt.tt * 2 * kHeadBM + static_cast<int>(rank) * kHeadBM;
+    if (threadIdx.x == 0) {
+      tiles[0] = pt.first;
+      tiles[1] = pt.end;
+      tiles[2] = pt.stride;
+      tiles[3] = pt.split;
+    }
+  }
 
   if (threadIdx.x == 0) {
     *abort_flag = 0;
@@ -667,21 +683,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kHeadThreads, 1)
     regs_decrease<kHeadCtlRegs>();
     if (warp == kHeadEpiWarps) {
       if (lane == 0) {
-        eval_producer<kTF32, kM>(p, base, row_base, rank, pt, abort_flag);
+        eval_producer<kTF32, kM>(p, base, row_base, rank, tiles, abort_flag);
         chain_trigger();
       }
     } else if (warp == kHeadEpiWarps + 1) {
       if (lane == 0 && rank == 0) {
         if constexpr (eval_slotted(kM))
-          eval_mma_slots<kTF32>(p, base, tmem, pt, abort_flag);
+          eval_mma_slots<kTF32>(p, base, tmem, tiles, abort_flag);
         else
-          eval_mma<kTF32, kM>(p, base, tmem, pt, abort_flag);
+          eval_mma<kTF32, kM>(p, base, tmem, tiles, abort_flag);
       }
       __syncwarp();
     }
   } else {
     regs_increase<kHeadEpiRegs>();
-    eval_epilogue<kM>(p, base, tmem, reinterpret_cast<float*>(gbase + Sm::kX), row_base, pt,
+    eval_epilogue<kM>(p, base, tmem, reinterpret_cast<float*>(gbase + Sm::kX), row_base, tiles,
                       warp, lane, abort_flag);
   }
 
