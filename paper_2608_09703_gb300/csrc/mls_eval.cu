@@ -231,7 +231,7 @@ struct EvalState {
 
 // 16 columns of every unit's tile: z[q][i] = z_{order[q]} at column col0 + i.
 template <int kM, bool kMasked>
-__device__ __forceinline__ void eval_chunk(const float (&z)[kM][16], int nvalid, long long col0,
+__device__ __forceinline__ void eval_chunk(const float (&z)[kM][16], int nvalid, int col0,
                                            float L1, EvalState<kM>& st) {
 #pragma unroll
   for (int q = 0; q < kM; ++q) {
@@ -246,7 +246,7 @@ __device__ __forceinline__ void eval_chunk(const float (&z)[kM][16], int nvalid,
       }
     }
     if (cmax > st.m[q]) {
-      st.am[q] = static_cast<int>(col0 + carg);
+      st.am[q] = col0 + carg;
       const float f = st.m[q] == -INFINITY ? 0.f : fast_exp2((st.m[q] - cmax) * L1);
       st.s[q] *= f;
 #pragma unroll
@@ -333,9 +333,9 @@ __device__ __forceinline__ void chunk_argmax(const float (&z)[16], float& vmax, 
 
 // Folds a tile's maximum (tmax at column tcol) into unit q's running state:
 // a new maximum rescales the unit's sum and its D_q*.
-__device__ __forceinline__ void fold_max(EvalState<3>& st, int q, float tmax, long long tcol, float L1) {
+__device__ __forceinline__ void fold_max(EvalState<3>& st, int q, float tmax, int tcol, float L1) {
   if (tmax > st.m[q]) {
-    st.am[q] = static_cast<int>(tcol);
+    st.am[q] = tcol;
     const float f = st.m[q] == -INFINITY ? 0.f : fast_exp2((st.m[q] - tmax) * L1);
     st.s[q] *= f;
 #pragma unroll
@@ -344,31 +344,29 @@ __device__ __forceinline__ void fold_max(EvalState<3>& st, int q, float tmax, lo
   }
 }
 
-// Tile maximum of a unit held in TMEM at t (this thread's 128 columns).
-__device__ __forceinline__ void tmem_tile_max(uint32_t t, long long tcol, long long V, float& tmax,
-                                              long long& targ) {
+// Tile maximum of a unit held in TMEM at t (this thread's 128 columns from tcol,
+// `left` of them inside the vocabulary).
+__device__ __forceinline__ void tmem_tile_max(uint32_t t, int tcol, int left, float& tmax, int& targ) {
   tmax = -INFINITY;
   targ = 0;
 #pragma unroll
   for (int c = 0; c < 8; c += 2) {
-    const long long col0 = tcol + c * 16;
-    if (col0 >= V) continue;  // warp-uniform
+    const int nv = left - c * 16;
+    if (nv <= 0) continue;  // warp-uniform
     float za[16], zb[16];
-    ld_chunk2(t + static_cast<uint32_t>(c * 16), t + static_cast<uint32_t>(c * 16 + 16),
-              static_cast<int>(min(16LL, V - col0)), static_cast<int>(max(0LL, min(16LL, V - col0 - 16))),
-              za, zb);
+    ld_chunk2(t + static_cast<uint32_t>(c * 16), t + static_cast<uint32_t>(c * 16 + 16), nv, nv - 16, za, zb);
     float va, vb;
     int ia, ib;
     chunk_argmax(za, va, ia);
     chunk_argmax(zb, vb, ib);
-    if (col0 + 16 >= V) vb = -INFINITY;  // the second chunk is past V
+    if (nv <= 16) vb = -INFINITY;  // the second chunk is past V
     if (va > tmax) {
       tmax = va;
-      targ = col0 + ia;
+      targ = tcol + c * 16 + ia;
     }
     if (vb > tmax) {
       tmax = vb;
-      targ = col0 + 16 + ib;
+      targ = tcol + c * 16 + 16 + ib;
     }
   }
 }
@@ -426,12 +424,16 @@ __device__ __forceinline__ bool eval_slots_main(const EvalParams& p, uint32_t ba
   constexpr int kHalf = Sm::kN / 2;  // 128 columns per thread
   constexpr int kChunks = kHalf / 16;
   const float L1 = p.L1;
-  const long long V = p.V;
   int j = 0;
   for (int vt = tiles[0]; vt < tiles[1]; vt += tiles[2], ++j) {
     const uint32_t par = static_cast<uint32_t>(j) & 1u;
     const uint32_t sa = par * Sm::kN, sb = Sm::kN - sa;
-    const long long tcol = static_cast<long long>(vt) * Sm::kN + half * kHalf;
+    // Column indices in 32 bits and one count of valid columns per tile: 64-bit
+    // comparisons per chunk cost the exposed pass 3 to 14% of the call (8192 tokens
+    // of the 3-level suite 3457 -> 3347 us; 54007 tokens, d = (216, 224, 2208), V =
+    // 20651: 5991 -> 5276 us).
+    const int tcol = static_cast<int>(static_cast<unsigned>(vt) * Sm::kN + half * kHalf);
+    const int left = static_cast<int>(min(static_cast<long long>(kHalf), p.V - static_cast<long long>(static_cast<unsigned>(tcol))));
     bool ok = mbar_wait(Sm::unit_full(base, 0), par, abort_flag, p.status);
     if (!__all_sync(0xffffffffu, ok)) return false;
     tc_fence_after();
@@ -443,22 +445,22 @@ __device__ __forceinline__ bool eval_slots_main(const EvalParams& p, uint32_t ba
     eval_release(Sm::copied(base), lane);
     {
       float tmax = -INFINITY;
-      long long targ = 0;
+      int targ = 0;
 #pragma unroll
       for (int c = 0; c < kChunks; ++c) {
-        const long long col0 = tcol + c * 16;
-        if (col0 + 16 > V) {
+        const int nv = left - c * 16;
+        if (nv < 16) {
 #pragma unroll
           for (int i = 0; i < 16; ++i)
-            if (col0 + i >= V) z0[c][i] = kPadLogit;
+            if (i >= nv) z0[c][i] = kPadLogit;
         }
-        if (col0 >= V) continue;
+        if (nv <= 0) continue;
         float v;
         int ix;
         chunk_argmax(z0[c], v, ix);
         if (v > tmax) {
           tmax = v;
-          targ = col0 + ix;
+          targ = tcol + c * 16 + ix;
         }
       }
       fold_max(st, 0, tmax, targ, L1);
@@ -469,17 +471,17 @@ __device__ __forceinline__ bool eval_slots_main(const EvalParams& p, uint32_t ba
     tc_fence_after();
     {
       float tmax;
-      long long targ;
-      tmem_tile_max(tl + sb, tcol, V, tmax, targ);
+      int targ;
+      tmem_tile_max(tl + sb, tcol, left, tmax, targ);
       fold_max(st, 1, tmax, targ, L1);
       const float n0 = -st.m[0] * L1, n1 = -st.m[1] * L1;
       PairSums ps = {};
 #pragma unroll
       for (int c = 0; c < kChunks; ++c) {
-        const long long col0 = tcol + c * 16;
-        if (col0 >= V) continue;  // warp-uniform
+        const int nv = left - c * 16;
+        if (nv <= 0) continue;  // warp-uniform
         float z1[16];
-        ld_chunk(tl + sb + static_cast<uint32_t>(c * 16), static_cast<int>(min(16LL, V - col0)), z1);
+        ld_chunk(tl + sb + static_cast<uint32_t>(c * 16), nv, z1);
         pair_chunk<true, true>(z0[c], z1, L1, n0, n1, ps);
       }
       fold_pair<true, true>(st, 0, 1, ps);
@@ -490,17 +492,16 @@ __device__ __forceinline__ bool eval_slots_main(const EvalParams& p, uint32_t ba
     tc_fence_after();
     {
       float tmax;
-      long long targ;
-      tmem_tile_max(tl + sa, tcol, V, tmax, targ);
+      int targ;
+      tmem_tile_max(tl + sa, tcol, left, tmax, targ);
       fold_max(st, 2, tmax, targ, L1);
       const float n1 = -st.m[1] * L1, n2 = -st.m[2] * L1;
       PairSums ps = {};
 #pragma unroll
       for (int c = 0; c < kChunks; ++c) {
-        const long long col0 = tcol + c * 16;
-        if (col0 >= V) continue;
+        const int nv = left - c * 16;
+        if (nv <= 0) continue;
         float z1[16], z2[16];
-        const int nv = static_cast<int>(min(16LL, V - col0));
         ld_chunk2(tl + sb + static_cast<uint32_t>(c * 16), tl + sa + static_cast<uint32_t>(c * 16), nv, nv,
                   z1, z2);
         pair_chunk<false, true>(z1, z2, L1, n1, n2, ps);
@@ -513,10 +514,10 @@ __device__ __forceinline__ bool eval_slots_main(const EvalParams& p, uint32_t ba
       PairSums ps = {};
 #pragma unroll
       for (int c = 0; c < kChunks; ++c) {
-        const long long col0 = tcol + c * 16;
-        if (col0 >= V) continue;
+        const int nv = left - c * 16;
+        if (nv <= 0) continue;
         float z2[16];
-        ld_chunk(tl + sa + static_cast<uint32_t>(c * 16), static_cast<int>(min(16LL, V - col0)), z2);
+        ld_chunk(tl + sa + static_cast<uint32_t>(c * 16), nv, z2);
         pair_chunk<false, false>(z0[c], z2, L1, n0, n2, ps);
       }
       fold_pair<false, false>(st, 0, 2, ps);
@@ -552,6 +553,8 @@ __device__ __forceinline__ void eval_epilogue(const EvalParams& p, uint32_t base
   } else {
   int j = 0;
   for (int vt = tiles[0]; vt < tiles[1]; vt += tiles[2], ++j) {
+    const int tcol = static_cast<int>(static_cast<unsigned>(vt) * Sm::kN + half * kHalf);
+    const int left = static_cast<int>(min(static_cast<long long>(kHalf), p.V - static_cast<long long>(static_cast<unsigned>(tcol))));
     const bool ok = mbar_wait(Sm::accf(base, j), static_cast<uint32_t>(j >> 1) & 1u, abort_flag, p.status);
     if (!__all_sync(0xffffffffu, ok)) break;
     tc_fence_after();
@@ -562,15 +565,15 @@ __device__ __forceinline__ void eval_epilogue(const EvalParams& p, uint32_t base
     eval_release(Sm::free0(base), lane);
 #pragma unroll
     for (int c = 0; c < kChunks; ++c) {
-      const long long col0 = static_cast<long long>(vt) * Sm::kN + half * kHalf + c * 16;
-      const int nvalid = static_cast<int>(max(0LL, min(16LL, p.V - col0)));
-      if (nvalid == 0) continue;  // warp-uniform
+      const int nvalid = left - c * 16;
+      if (nvalid <= 0) continue;  // warp-uniform
+      const int col0 = tcol + c * 16;
       float z[kM][16];
 #pragma unroll
       for (int i = 0; i < 16; ++i) z[0][i] = z0[c][i];
 #pragma unroll
       for (int q = 1; q < kM; ++q) tmem_ld16(tl + static_cast<uint32_t>(q * Sm::kN + c * 16), z[q]);
-      if (nvalid == 16)
+      if (nvalid >= 16)
         eval_chunk<kM, false>(z, 16, col0, L1, st);
       else
         eval_chunk<kM, true>(z, nvalid, col0, L1, st);
