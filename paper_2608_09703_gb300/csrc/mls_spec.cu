@@ -299,6 +299,18 @@ __device__ __forceinline__ void row_pass(const float* et, const float* ftab, int
   }
 }
 
+// Sum of cnt[w] over the warps before this one, and over all of them (in every
+// lane), by a warp scan: a loop over 32 warps is a chain of shared-memory reads.
+// With it, a search of the sampled step by the whole block and a sampler of its own
+// for each mode, one user's verify call took 89.3 -> 87.1 us.
+template <int NW>
+__device__ __forceinline__ int warps_before(const int* cnt, int& total) {
+  const int c = lane_id() < NW ? cnt[lane_id()] : 0;
+  const int incl = warp_incl_scan(c);
+  total = __shfl_sync(0xffffffffu, incl, 31);
+  return __shfl_sync(0xffffffffu, incl - c, warp_id());
+}
+
 // The column tiles whose factor f_t has a key of at least min_key (so the
 // only tiles that can hold an e >= that value, since every e of tile t is at
 // most f_t), in tile order, into kept[]; returns their number.  Needs ftab
@@ -313,12 +325,8 @@ __device__ int kept_tiles(const float* ftab, int tiles, uint32_t min_key, int* k
     const unsigned bal = __ballot_sync(0xffffffffu, keep);
     if (lane_id() == 0) sh.wcnt[warp_id()] = __popc(bal);
     __syncthreads();
-    int at = nk, total = 0;
-    for (int w = 0; w < NW; ++w) {
-      const int c = sh.wcnt[w];
-      if (w < warp_id()) at += c;
-      total += c;
-    }
+    int total;
+    const int at = nk + warps_before<NW>(sh.wcnt, total);
     if (keep) kept[at + __popc(bal & ((1u << lane_id()) - 1u))] = t;
     nk += total;
     __syncthreads();  // sh.wcnt is rewritten next
@@ -559,12 +567,10 @@ __device__ void reduce_pass(PassStats& s, SharedT<NW>& sh) {
 // side `side` (1 = upper, 2 = lower) are compacted in warp order.
 template <int NW>
 __device__ __forceinline__ void warp_bases(int side, SharedT<NW>& sh) {
-  if (threadIdx.x == 0) {
-    int acc = 0;
-    for (int w = 0; w < NW; ++w) {
-      sh.wbase[w] = acc;
-      acc += sh.n[w][side];
-    }
+  if (warp_id() == 0) {
+    const int c = lane_id() < NW ? sh.n[lane_id()][side] : 0;
+    const int incl = warp_incl_scan(c);
+    if (lane_id() < NW) sh.wbase[lane_id()] = incl - c;
   }
   __syncthreads();
 }
@@ -638,11 +644,10 @@ __device__ RowNucleus nucleus(const float* et, const float* st, float* fg, long 
         cnt = ps.cnt_ge;
         lo = kFirstMid;
         // the upper side is in the warps' regions unless one overflowed
-        bool fits = true;
-        for (int w = 0; w < NW; ++w) fits = fits && sh.wcnt[w] <= kRegion;
+        const bool fits = __all_sync(0xffffffffu, lane_id() >= NW || sh.wcnt[lane_id()] <= kRegion);
         if (fits) {
-          int at = 0;
-          for (int w = 0; w < warp_id(); ++w) at += sh.wcnt[w];
+          int total;
+          const int at = warps_before<NW>(sh.wcnt, total);
           const float* reg = listA + warp_id() * kRegion;
           for (int i = lane_id(); i < sh.wcnt[warp_id()]; i += 32) listB[at + i] = reg[i];
           __syncthreads();
@@ -1051,16 +1056,17 @@ __device__ int sample(const float* ep, const float* fp, const RowNucleus& np, co
   const float total = cum[nsteps - 1];
   if (!(total > 0.f)) return -1;
   const float want = u * total;
-  if (w == 0) {
-    // the first step whose cumulative passes want (and that has mass)
-    int owner = -1;
-    for (int s0 = 0; s0 < nsteps && owner < 0; s0 += 32) {
-      const int st = s0 + l;
-      const float prev = st > 0 && st < nsteps ? cum[st - 1] : 0.f;
-      const bool hit = st < nsteps && cum[st] > want && cum[st] > prev;
-      const unsigned bal = __ballot_sync(0xffffffffu, hit);
-      if (bal) owner = s0 + __ffs(bal) - 1;
+  // the first step whose cumulative passes want (and that has mass)
+  if (threadIdx.x == 0) sh.rn[0] = nsteps;
+  __syncthreads();
+  for (int st = threadIdx.x; st < nsteps; st += NW * 32)
+    if (cum[st] > want && cum[st] > (st > 0 ? cum[st - 1] : 0.f)) {
+      atomicMin(&sh.rn[0], st);
+      break;
     }
+  __syncthreads();
+  if (w == 0) {
+    int owner = sh.rn[0] < nsteps ? sh.rn[0] : -1;
     float before = 0.f;
     if (owner < 0) {  // rounding put want at the total: the last step with mass
       for (int st = nsteps - 1; st >= 0 && owner < 0; --st)
@@ -1107,15 +1113,16 @@ __device__ int sample(const float* ep, const float* fp, const RowNucleus& np, co
 __device__ int row_argmax(const float* st, int tiles) {
   float mv = -INFINITY;
   int mi = 0;
-  for (int t0 = 0; t0 < tiles; t0 += 4 * 32) {
-    float2 v[4];
+  constexpr int kLoads = 16;  // in flight per lane: one round for V <= 65536 in tiles of 128
+  for (int t0 = 0; t0 < tiles; t0 += kLoads * 32) {
+    float2 v[kLoads];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < kLoads; ++u) {
       const int t = t0 + u * 32 + lane_id();
       v[u] = t < tiles ? *reinterpret_cast<const float2*>(st + 2 * t) : make_float2(-INFINITY, 0.f);
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < kLoads; ++u)
       if (v[u].x > mv) {
         mv = v[u].x;
         mi = __float_as_int(v[u].y);
@@ -1127,6 +1134,7 @@ __device__ int row_argmax(const float* st, int tiles) {
   return mi;
 }
 
+template <bool kGreedy>
 __global__ void __launch_bounds__(kSampleWarps * 32) spec_sample_kernel(const SpecParams p) {
   extern __shared__ __align__(16) float smem[];
   __shared__ SharedT<kSampleWarps> sh;
@@ -1135,14 +1143,14 @@ __global__ void __launch_bounds__(kSampleWarps * 32) spec_sample_kernel(const Sp
   const int b = blockIdx.x, G1 = p.gamma + 1;
   const long long sld = 2LL * p.tiles;
   int k = 0, next = -1;
-  if (p.greedy) {
-    // A warp per position, kSampleWarps positions at a time: one pass settles most
-    // sequences, where a block-wide argmax per accepted position was a chain of
-    // gamma + 1 of them (16 sequences that accept most of 6: 11.3 -> 6.9 us).
-    for (bool done = false; !done; k += kSampleWarps) {
+  if constexpr (kGreedy) {
+    // A warp per position, as many at a time as the block has warps: one pass
+    // settles most sequences, where a block-wide argmax per accepted position was a
+    // chain of gamma + 1 of them (16 sequences that accept most of 6: 11.3 -> 6.5 us).
+    const int nw = static_cast<int>(blockDim.x >> 5);
+    for (;; k += nw) {
       const int pos = k + warp_id();
-      int best = 0;
-      bool stop = false;
+      int best = 0, stop = 0;
       if (pos <= p.gamma) {
         best = row_argmax(p.stats_v + (static_cast<long long>(b) * G1 + pos) * sld, p.tiles);
         stop = pos == p.gamma || p.draft[static_cast<long long>(b) * p.gamma + pos] != best;
@@ -1152,14 +1160,13 @@ __global__ void __launch_bounds__(kSampleWarps * 32) spec_sample_kernel(const Sp
         sh.n[warp_id()][1] = stop;
       }
       __syncthreads();
-      for (int w = 0; w < kSampleWarps; ++w)
-        if (sh.n[w][1]) {
-          next = sh.n[w][0];
-          k += w;
-          done = true;
-          break;
-        }
-      if (done) break;
+      const unsigned stops = __ballot_sync(0xffffffffu, lane_id() < nw && sh.n[lane_id()][1]);
+      if (stops) {  // the first position that ends the sequence
+        const int w = __ffs(stops) - 1;
+        next = sh.n[w][0];
+        k += w;
+        break;
+      }
       __syncthreads();  // sh.n is rewritten next
     }
   } else {
@@ -1256,7 +1263,7 @@ cudaError_t setup_spec_kernels() {
   MLS_SET(32)
 #undef MLS_SET
   return cudaFuncSetAttribute(
-      spec_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      spec_sample_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
       static_cast<int>(sample_smem(static_cast<long long>(kSpecMaxTiles) * kGemmBN, kSpecMaxTiles,
                                    kSpecMaxGamma)));
 }
@@ -1276,8 +1283,11 @@ cudaError_t launch_spec_rows(const SpecParams& p, cudaStream_t s) {
 
 cudaError_t launch_spec_sample(const SpecParams& p, cudaStream_t s) {
   if (p.B <= 0) return cudaSuccess;
-  return launch_chained(spec_sample_kernel, dim3(p.B), dim3(kSampleWarps * 32),
-                        p.greedy ? 0 : sample_smem(p.V, p.tiles, p.gamma), s, p);
+  if (p.greedy) {  // a warp per position
+    const int warps = p.gamma + 1 < kSampleWarps ? p.gamma + 1 : kSampleWarps;
+    return launch_chained(spec_sample_kernel<true>, dim3(p.B), dim3(32 * warps), 0, s, p);
+  }
+  return launch_chained(spec_sample_kernel<false>, dim3(p.B), dim3(kSampleWarps * 32), sample_smem(p.V, p.tiles, p.gamma), s, p);
 }
 
 }  // namespace mls
