@@ -346,7 +346,7 @@ def gpu_arm(args, rank, world, local):
     wl = workload(args)
     H, W, y = synth.make_inputs(wl, seed=1234 + rank, device=dev)
     op = B.HeadLoss(wl.d, wl.T, wl.V, teacher=wl.teacher_index, tau=wl.tau, alpha=wl.alpha,
-                    w=wl.weights, dtype=torch.bfloat16, device=dev, vocab_group=args.vocab_group)
+                    w=wl.weights, dtype=H[0].dtype, device=dev, vocab_group=args.vocab_group)
 
     nvtx = torch.cuda.nvtx
 
