@@ -67,6 +67,14 @@ struct Vec<float> {
 };
 
 __device__ __forceinline__ uint4 ld16(const void* p) { return *reinterpret_cast<const uint4*>(p); }
+// The streaming kernels' loads: read-only, so that the compiler issues the loads of
+// several vectors ahead of the stores between them (with plain loads every store
+// ended the run).  Each element is still read before the same thread overwrites it.
+// Forward and backward: 2000 fp32 tokens of 3000 + 5192 channels 136.3 -> 98.9 us;
+// backward of 16384 bf16 tokens of 6144 + 2048 202.7 -> 195.4 us, of 714 24.5 -> 20.6.
+__device__ __forceinline__ uint4 ld16_stream(const void* p) {
+  return __ldg(static_cast<const uint4*>(p));
+}
 __device__ __forceinline__ void st16(void* p, const uint4& v) { *reinterpret_cast<uint4*>(p) = v; }
 
 // Tells the compiler the cached vectors may have changed, so it re-unpacks
@@ -115,7 +123,7 @@ __device__ __forceinline__ float sumsq_stream(const E* row, int n, int lane) {
   float acc = 0.f;
   for (int k = lane * N; k < n; k += 32 * N) {
     float f[N];
-    Vec<E>::unpack(ld16(row + k), f);
+    Vec<E>::unpack(ld16_stream(row + k), f);
 #pragma unroll
     for (int i = 0; i < N; ++i) acc = fmaf(f[i], f[i], acc);
   }
@@ -184,12 +192,12 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock) junction_fwd_kernel(const 
     const float s = no > 0.f ? ne / no : 0.f;
     for (int k = lane * N; k < p.d_prev; k += 32 * N) {
       float f[N];
-      Vec<E>::unpack(ld16(o + k), f);
+      Vec<E>::unpack(ld16_stream(o + k), f);
 #pragma unroll
       for (int i = 0; i < N; ++i) f[i] *= s;
       st16(xo + k, Vec<E>::pack(f));
     }
-    for (int k = lane * N; k < r.de; k += 32 * N) st16(xe + k, ld16(e + k));
+    for (int k = lane * N; k < r.de; k += 32 * N) st16(xe + k, ld16_stream(e + k));
   }
 }
 
@@ -263,8 +271,8 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock) junction_bwd_kernel(const 
   } else {
     for (int k = lane * N; k < p.d_prev; k += 32 * N) {
       float fo[N], fg[N];
-      Vec<E>::unpack(ld16(o + k), fo);
-      Vec<E>::unpack(ld16(go + k), fg);
+      Vec<E>::unpack(ld16_stream(o + k), fo);
+      Vec<E>::unpack(ld16_stream(go + k), fg);
 #pragma unroll
       for (int i = 0; i < N; ++i) {
         oo = fmaf(fo[i], fo[i], oo);
@@ -280,16 +288,16 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock) junction_bwd_kernel(const 
     const float ce = (no > 0.f && ee > 0.f) ? s * dot / ee : 0.f;
     for (int k = lane * N; k < p.d_prev; k += 32 * N) {
       float fo[N], fg[N], r[N];
-      Vec<E>::unpack(ld16(o + k), fo);
-      Vec<E>::unpack(ld16(go + k), fg);
+      Vec<E>::unpack(ld16_stream(o + k), fo);
+      Vec<E>::unpack(ld16_stream(go + k), fg);
 #pragma unroll
       for (int i = 0; i < N; ++i) r[i] = s * fmaf(-fo[i], co, fg[i]);
       st16(d_o + k, Vec<E>::pack(r));
     }
     for (int k = lane * N; k < de; k += 32 * N) {
       float fe[N], fg[N], r[N];
-      Vec<E>::unpack(ld16(e + k), fe);
-      Vec<E>::unpack(ld16(ge + k), fg);
+      Vec<E>::unpack(ld16_stream(e + k), fe);
+      Vec<E>::unpack(ld16_stream(ge + k), fg);
 #pragma unroll
       for (int i = 0; i < N; ++i) r[i] = fmaf(ce, fe[i], fg[i]);
       st16(d_e + k, Vec<E>::pack(r));
