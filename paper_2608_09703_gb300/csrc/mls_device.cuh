@@ -48,11 +48,16 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 // ---------------------------------------------------------------- dependent launches
 // The kernels of one call run as a chain of programmatic dependent launches
 // (launch_chained): a kernel lets its successor be scheduled once its CTAs have
-// issued their last loads (chain_trigger; small kernels do so at once), and before it touches what a predecessor writes,
-// or writes what one reads, it waits until its predecessor has completed
-// (chain_wait), which that one does only after its own.  Every kernel launched
-// that way waits in some thread of each CTA.  A call's first kernel is launched
-// normally, so whatever ran on the stream before the call is complete.
+// issued their last loads (chain_trigger; small kernels do so at once), and
+// before it touches what a predecessor writes, or writes what one reads, it
+// waits until its predecessor has completed (chain_wait), which that one does
+// only after its own.  Every kernel launched that way waits in some thread of
+// each CTA.  A call's first kernel is launched normally, so whatever ran on the
+// stream before the call is complete.
+// The read-only path (__ldg, const __restrict__) is for what nobody writes while
+// the kernel runs, so in a chained kernel only for the caller's own inputs: what
+// the kernels of the same call hand on is read with plain loads, which stay
+// behind the wait.
 // Measured, unchained against chained: a step of 256 fp32 tokens, d = (128, 256),
 // V = 1024: 72.7 -> 61.4 us; 3000 tokens, d = (264, 712), V = 5000: 176 -> 164 us;
 // pairwise evaluation of 50 tokens 24.6 -> 20.6 us; one user's verify call 91.6

@@ -89,6 +89,10 @@ __device__ __forceinline__ float warp_incl_scan(float v) {
   return v;
 }
 
+// Four stored probabilities.  A plain load: the launch that writes them may still be
+// running when these kernels start (chain_wait), which rules out the read-only path.
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+
 __device__ __forceinline__ float comp(const float4& v, int j) {
   return j == 0 ? v.x : j == 1 ? v.y : j == 2 ? v.z : v.w;
 }
@@ -213,7 +217,7 @@ __device__ __forceinline__ void for_row(const float* et, const float* ftab, int 
     for (int u = 0; u < kUnroll; ++u) {
       const long long i0 = base + u * kStride + l * 4;
       v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (i0 < V) v[u] = __ldg(reinterpret_cast<const float4*>(et + i0));
+      if (i0 < V) v[u] = ld4(et + i0);
     }
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
@@ -275,7 +279,7 @@ __device__ __forceinline__ void row_pass(const float* et, const float* ftab, int
       const int s0 = base + u * kStride, i0 = s0 + l * 4;
       // a tile whose maximum lies below the bracket holds no candidate
       const bool live = s0 < V && __float_as_uint(ftab[s0 >> tsh]) >= lo;
-      v[u] = live && i0 < V ? __ldg(reinterpret_cast<const float4*>(et + i0))
+      v[u] = live && i0 < V ? ld4(et + i0)
                             : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 #pragma unroll
@@ -367,7 +371,7 @@ __device__ __forceinline__ void first_pass(const float* et, const float* ftab, i
         const int t = kept[q >> sub];
         fm[u] = ftab[t];
         i0s[u] = (t << tsh) + (q & ((1 << sub) - 1)) * kStep + l * 4;
-        if (i0s[u] < V) v[u] = __ldg(reinterpret_cast<const float4*>(et + i0s[u]));
+        if (i0s[u] < V) v[u] = ld4(et + i0s[u]);
       }
     }
 #pragma unroll
@@ -436,7 +440,7 @@ __device__ void octave_pass(const float* et, const float* ftab, int tsh, int V, 
       const int s0 = base + u * kStride, i0 = s0 + l * 4;
       fm[u] = s0 < V ? ftab[s0 >> tsh] : 0.f;  // warp-uniform
       v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (__float_as_uint(fm[u]) >= lo && i0 < V) v[u] = __ldg(reinterpret_cast<const float4*>(et + i0));
+      if (__float_as_uint(fm[u]) >= lo && i0 < V) v[u] = ld4(et + i0);
     }
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
@@ -480,7 +484,7 @@ __device__ __forceinline__ void row_compact(const float* et, const float* ftab, 
       const int s0 = base + u * kStride, i0 = s0 + l * 4;
       fm[u] = s0 < V ? ftab[s0 >> tsh] : 0.f;  // warp-uniform
       v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (__float_as_uint(fm[u]) >= lo && i0 < V) v[u] = __ldg(reinterpret_cast<const float4*>(et + i0));
+      if (__float_as_uint(fm[u]) >= lo && i0 < V) v[u] = ld4(et + i0);
     }
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
@@ -909,7 +913,7 @@ __device__ __forceinline__ float4 load_e(const float* et, const float* ftab, int
                                          long long V) {
   float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
   if (i0 < V) {
-    v = __ldg(reinterpret_cast<const float4*>(et + i0));
+    v = ld4(et + i0);
     const float fm = ftab[i0 >> tsh];
     v.x *= fm;
     v.y *= fm;
