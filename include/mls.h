@@ -151,7 +151,8 @@ int mls_head_pairwise(const mls_problem* p, const void* const* H, const void* co
  * are overwritten (same storage type) with
  *   dL/do = s (g_o - o (g_o . o) / ||o||^2),  dL/de = g_e + s (g_o . o) e / ||e||^2,
  *   s = ||e|| / ||o||  (both terms 0 when ||o|| = 0).
- * Asynchronous on `stream`; returns 0 or a negative MLS_ERR_* code.
+ * d_o may be the buffer o and d_e the buffer e; otherwise outputs do not overlap
+ * inputs.  Asynchronous on `stream`; returns 0 or a negative MLS_ERR_* code.
  */
 int mls_junction_fwd(int64_t T, int32_t d_prev, int32_t d_next, int32_t in_dtype,
                      int32_t embed_first, const void* o, const void* e, void* x,

@@ -67,14 +67,6 @@ struct Vec<float> {
 };
 
 __device__ __forceinline__ uint4 ld16(const void* p) { return *reinterpret_cast<const uint4*>(p); }
-// The streaming kernels' loads: read-only, so that the compiler issues the loads of
-// several vectors ahead of the stores between them (with plain loads every store
-// ended the run).  Each element is still read before the same thread overwrites it.
-// Forward and backward: 2000 fp32 tokens of 3000 + 5192 channels 136.3 -> 98.9 us;
-// backward of 16384 bf16 tokens of 6144 + 2048 202.7 -> 195.4 us, of 714 24.5 -> 20.6.
-__device__ __forceinline__ uint4 ld16_stream(const void* p) {
-  return __ldg(static_cast<const uint4*>(p));
-}
 __device__ __forceinline__ void st16(void* p, const uint4& v) { *reinterpret_cast<uint4*>(p) = v; }
 
 // Tells the compiler the cached vectors may have changed, so it re-unpacks
@@ -117,16 +109,60 @@ __device__ __forceinline__ float sumsq_cached(const uint4 (&v)[R]) {
   return acc;
 }
 
+// The streaming kernels walk a segment (or two side by side) a batch of vectors
+// per lane at a time: the batch's loads are issued before anything is done with
+// them, since the stores of one vector would otherwise hold back the loads of
+// the next.  They are plain loads, and every element is read before the same
+// thread overwrites it, so a gradient may take the place of its input.  Batches
+// of 8 fp32 or 4 bf16 vectors, half as many of two segments, against read-only
+// loads that the compiler scheduled (which forbid in-place gradients): forward
+// and backward of 2000 fp32 tokens of 3000 + 5192 channels 100 -> 76 us, 16384:
+// 590 -> 569; 2000 bf16 tokens of 4000 + 12000 101 -> 91, 16384: 573 -> 548.  The
+// fp32 backward's 64 registers leave 8 blocks per SM, so that 5300 tokens have a
+// short second wave (125 -> 133 us).
+template <typename E>
+constexpr int kBatch = 32 / Vec<E>::N;
+
+template <typename E, typename F>
+__device__ __forceinline__ void stream(const E* a, int n, int lane, F&& f) {
+  constexpr int N = Vec<E>::N, kStep = 32 * N, kB = kBatch<E>;
+  for (int k0 = lane * N; k0 < n; k0 += kB * kStep) {
+    uint4 va[kB];
+#pragma unroll
+    for (int u = 0; u < kB; ++u)
+      if (k0 + u * kStep < n) va[u] = ld16(a + k0 + u * kStep);
+#pragma unroll
+    for (int u = 0; u < kB; ++u)
+      if (k0 + u * kStep < n) f(k0 + u * kStep, va[u]);
+  }
+}
+template <typename E, typename F>
+__device__ __forceinline__ void stream(const E* a, const E* b, int n, int lane, F&& f) {
+  constexpr int N = Vec<E>::N, kStep = 32 * N, kB = kBatch<E> / 2;
+  for (int k0 = lane * N; k0 < n; k0 += kB * kStep) {
+    uint4 va[kB], vb[kB];
+#pragma unroll
+    for (int u = 0; u < kB; ++u)
+      if (k0 + u * kStep < n) {
+        va[u] = ld16(a + k0 + u * kStep);
+        vb[u] = ld16(b + k0 + u * kStep);
+      }
+#pragma unroll
+    for (int u = 0; u < kB; ++u)
+      if (k0 + u * kStep < n) f(k0 + u * kStep, va[u], vb[u]);
+  }
+}
+
 template <typename E>
 __device__ __forceinline__ float sumsq_stream(const E* row, int n, int lane) {
   constexpr int N = Vec<E>::N;
   float acc = 0.f;
-  for (int k = lane * N; k < n; k += 32 * N) {
+  stream(row, n, lane, [&](int, const uint4& v) {
     float f[N];
-    Vec<E>::unpack(ld16_stream(row + k), f);
+    Vec<E>::unpack(v, f);
 #pragma unroll
     for (int i = 0; i < N; ++i) acc = fmaf(f[i], f[i], acc);
-  }
+  });
   return acc;
 }
 
@@ -190,14 +226,14 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock) junction_fwd_kernel(const 
     const float no = sqrtf(warp_sum(sumsq_stream(o, p.d_prev, lane)));
     const float ne = sqrtf(warp_sum(sumsq_stream(e, r.de, lane)));
     const float s = no > 0.f ? ne / no : 0.f;
-    for (int k = lane * N; k < p.d_prev; k += 32 * N) {
+    stream(o, p.d_prev, lane, [&](int k, const uint4& v) {
       float f[N];
-      Vec<E>::unpack(ld16_stream(o + k), f);
+      Vec<E>::unpack(v, f);
 #pragma unroll
       for (int i = 0; i < N; ++i) f[i] *= s;
       st16(xo + k, Vec<E>::pack(f));
-    }
-    for (int k = lane * N; k < r.de; k += 32 * N) st16(xe + k, ld16_stream(e + k));
+    });
+    stream(e, r.de, lane, [&](int k, const uint4& v) { st16(xe + k, v); });
   }
 }
 
@@ -269,16 +305,16 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock) junction_bwd_kernel(const 
       }
     }
   } else {
-    for (int k = lane * N; k < p.d_prev; k += 32 * N) {
+    stream(o, go, p.d_prev, lane, [&](int, const uint4& v, const uint4& vg) {
       float fo[N], fg[N];
-      Vec<E>::unpack(ld16_stream(o + k), fo);
-      Vec<E>::unpack(ld16_stream(go + k), fg);
+      Vec<E>::unpack(v, fo);
+      Vec<E>::unpack(vg, fg);
 #pragma unroll
       for (int i = 0; i < N; ++i) {
         oo = fmaf(fo[i], fo[i], oo);
         dot = fmaf(fg[i], fo[i], dot);
       }
-    }
+    });
     oo = warp_sum(oo);
     dot = warp_sum(dot);
     ee = warp_sum(sumsq_stream(e, de, lane));
@@ -286,22 +322,22 @@ __global__ void __launch_bounds__(32 * kRowsPerBlock) junction_bwd_kernel(const 
     const float s = no > 0.f ? ne / no : 0.f;
     const float co = no > 0.f ? dot / oo : 0.f;
     const float ce = (no > 0.f && ee > 0.f) ? s * dot / ee : 0.f;
-    for (int k = lane * N; k < p.d_prev; k += 32 * N) {
+    stream(o, go, p.d_prev, lane, [&](int k, const uint4& v, const uint4& vg) {
       float fo[N], fg[N], r[N];
-      Vec<E>::unpack(ld16_stream(o + k), fo);
-      Vec<E>::unpack(ld16_stream(go + k), fg);
+      Vec<E>::unpack(v, fo);
+      Vec<E>::unpack(vg, fg);
 #pragma unroll
       for (int i = 0; i < N; ++i) r[i] = s * fmaf(-fo[i], co, fg[i]);
       st16(d_o + k, Vec<E>::pack(r));
-    }
-    for (int k = lane * N; k < de; k += 32 * N) {
+    });
+    stream(e, ge, de, lane, [&](int k, const uint4& v, const uint4& vg) {
       float fe[N], fg[N], r[N];
-      Vec<E>::unpack(ld16_stream(e + k), fe);
-      Vec<E>::unpack(ld16_stream(ge + k), fg);
+      Vec<E>::unpack(v, fe);
+      Vec<E>::unpack(vg, fg);
 #pragma unroll
       for (int i = 0; i < N; ++i) r[i] = fmaf(ce, fe[i], fg[i]);
       st16(d_e + k, Vec<E>::pack(r));
-    }
+    });
   }
 }
 

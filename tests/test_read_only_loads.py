@@ -38,3 +38,9 @@ def test_chained_kernels_read_only_the_callers_inputs_that_way():
             assert any(re.match(r"\W*(?:reinterpret_cast<[^>]*>\()?" + ok, operand)
                        for ok in INPUTS.get(name, ())), f"{name}: {operand}"
     assert seen >= 4
+
+
+def test_junction_loads_allow_gradients_over_inputs():
+    """d_o may be o and d_e may be e, so nothing the junction reads stays unwritten."""
+    with open(os.path.join(CSRC, "mls_junction.cu")) as f:
+        assert list(read_only_operands(f.read())) == []
