@@ -446,6 +446,26 @@ Plan make_plan(const mls_problem* p, int pairs, int gemm_pairs) {
   return pl;
 }
 
+// One vocabulary group of the backward: its columns and how its two launches are cut.
+struct GroupPlan {
+  long long c0 = 0, cols = 0;
+  TileSplit split = {};  // the head kernel's vocabulary tiles
+  GemmCut cut;
+};
+
+GroupPlan plan_group(const mls_problem* p, const Plan& pl, long long g, int pairs, int gemm_pairs) {
+  GroupPlan gp;
+  gp.c0 = g * pl.group;
+  gp.cols = (p->V - gp.c0 < pl.group) ? p->V - gp.c0 : pl.group;
+  const int vt0 = static_cast<int>(gp.c0 / kHeadBN);
+  gp.split = choose_splits(pl.ntt, ceil_div(gp.c0 + gp.cols, kHeadBN) - vt0, pairs, pl.band_bwd);
+  gp.split.begin += vt0;
+  gp.split.main_end += vt0;
+  gp.split.end += vt0;
+  gp.cut = cut_gemm(p->M, p->d, p->T, gp.cols, g == 0, 128 / pl.elt, gemm_pairs);
+  return gp;
+}
+
 bool aligned16(const void* ptr) { return (reinterpret_cast<uintptr_t>(ptr) & 15u) == 0; }
 
 // 2-D row-major tensor [rows, cols] of `elt`-byte elements (128-byte swizzle
@@ -573,6 +593,28 @@ extern "C" size_t mls_workspace_size(const mls_problem* p) {
   return make_plan(p, head, gemm).total;
 }
 
+// How a problem's launches are cut, for tests that have to know which path a shape
+// takes (not part of mls.h): out[0..5] = backward groups, partial-state slots of the
+// forward and of the evaluation, extra pairs per token tile of both, bytes of the
+// copies of split reductions; then per group of the backward the extra pairs, whether
+// dH runs in wide units, and the units that share a long reduction.  Writes at most n
+// values, returns how many there are or a negative MLS_ERR_* code.
+extern "C" int mls_test_plan(const mls_problem* p, int64_t* out, int n) {
+  const int rc = validate(p);
+  if (rc) return rc;
+  int head = 0, gemm = 0;
+  current_pairs(head, gemm);
+  const Plan pl = make_plan(p, head, gemm);
+  std::vector<int64_t> v = {pl.ngroups,          pl.nparts, pl.eval_nparts, pl.split.extra,
+                            pl.eval_split.extra, static_cast<int64_t>(pl.bwd_bytes - pl.off_split)};
+  for (long long g = 0; g < pl.ngroups && static_cast<int>(v.size()) < n; ++g) {
+    const GroupPlan gp = plan_group(p, pl, g, head, gemm);
+    v.insert(v.end(), {gp.split.extra, gp.cut.wide ? 1 : 0, gp.cut.ksplit});
+  }
+  for (size_t i = 0; i < v.size() && static_cast<int>(i) < n; ++i) out[i] = v[i];
+  return static_cast<int>(6 + 3 * pl.ngroups);
+}
+
 extern "C" int mls_head_loss_fwd(const mls_problem* p, const void* const* H, const void* const* W,
                                  const int32_t* targets, float* loss, float* tok_loss,
                                  float* tok_diag, int32_t* argmax, float* stats, void* ws,
@@ -685,21 +727,16 @@ extern "C" int mls_head_loss_bwd(const mls_problem* p, const void* const* H, con
       return MLS_ERR_CUDA;
   }
 
-  const long long tiles_per_group = pl.group / kHeadBN;
   for (long long g = 0; g < pl.ngroups; ++g) {
-    const long long c0 = g * pl.group;
-    const long long gc = (p->V - c0 < pl.group) ? p->V - c0 : pl.group;  // columns of this group
-    const int vt0 = static_cast<int>(g * tiles_per_group);
-    hp.split = choose_splits(pl.ntt, ceil_div(c0 + gc, kHeadBN) - vt0, dev->head_pairs, pl.band_bwd);
-    hp.split.begin += vt0;
-    hp.split.main_end += vt0;
-    hp.split.end += vt0;
+    const GroupPlan gp = plan_group(p, pl, g, dev->head_pairs, dev->gemm_pairs);
+    const long long c0 = gp.c0, gc = gp.cols;
+    hp.split = gp.split;
     hp.g_col0 = c0;
     if ((rc = timed("head_bwd", s, [&] { return launch_head_bwd(hp, tf32, p->tau == 1.0f, s); }))) return rc;
     // dW and dH of every sub-model in one persistent launch, the class with the
     // longer reduction (dH: the group's columns, dW: T) first.
     const int pairs = dev->gemm_pairs, M = p->M;
-    const GemmCut cut = cut_gemm(M, p->d, p->T, gc, g == 0, KE, pairs);
+    const GemmCut& cut = gp.cut;
     float* split_ws = reinterpret_cast<float*>(wsb + pl.off_split);
     SplitSumParams sum;
     std::memset(&sum, 0, sizeof sum);

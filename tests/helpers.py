@@ -8,14 +8,34 @@ the fp64 oracle using the tolerances stated for this operation:
 """
 from __future__ import annotations
 
+import ctypes
+import os
+
 import numpy as np
 import torch
 
 from paper_2608_09703_gb300 import binding as B
+from paper_2608_09703_gb300 import build as mbuild
 from paper_2608_09703_gb300 import synth
 
 LOSS_RTOL = 1e-3
 GRAD_TOL = 2e-2
+
+
+def launch_plan(wl, vocab_group=0):
+    """How the library cuts a workload's launches (mls_test_plan): which path a shape takes."""
+    p = B.Problem(wl.d, wl.T, wl.V, wl.teacher_index, wl.tau, wl.alpha, wl.weights,
+                  B.MLS_BF16 if wl.dtype == "bf16" else B.MLS_FP32, vocab_group)
+    if not os.path.exists(B.library_path()):
+        mbuild.build()
+    out = (ctypes.c_int64 * 96)()
+    n = B.lib().mls_test_plan(p.ref(), out, len(out))
+    assert 9 <= n <= len(out), n
+    keys = ("groups", "fwd_parts", "eval_parts", "fwd_extra", "eval_extra", "split_bytes")
+    plan = dict(zip(keys, out))
+    for k, name in enumerate(("bwd_extra", "wide", "ksplit")):
+        plan[name] = [out[i] for i in range(6 + k, n, 3)]
+    return plan
 
 
 def run_gpu(wl: synth.Workload, H, W, y, grad_scale=1.0, vocab_group=0, backward=True):

@@ -32,7 +32,7 @@ def grads_match_oracle(wl, seed, vocab_group=0):
 @pytest.mark.parametrize("T,d,V,vocab_group", [
     (300, (36, 100), 1003, 0),       # widths, tokens and vocabulary that end inside a 32-wide block
     (257, (256, 516), 700, 256),     # three vocabulary groups, dH accumulated
-    (40, (512, 1024), 17000, 0),     # dH over more than 512 k-blocks of 32: wide units
+    (40, (512, 1024), 17000, 0),     # dH over more than 512 k-blocks of 32, 7 units each
 ])
 def test_fp32_reads_g_h_w_in_place(T, d, V, vocab_group):
     """fp32 storage: both products read G, H and W transposed or not where they

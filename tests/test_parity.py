@@ -10,7 +10,7 @@ from oracle import oracle
 from paper_2608_09703_gb300 import binding as B
 from paper_2608_09703_gb300 import synth
 
-from helpers import check_forward, check_grads, exact_logits, rel_close, run_gpu
+from helpers import check_forward, check_grads, exact_logits, launch_plan, rel_close, run_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -61,15 +61,14 @@ def test_vocab_groups_match(vocab_group):
     full_parity(wl, H, W, y, vocab_group=vocab_group)
 
 
-@pytest.mark.parametrize("T,V,vocab_group", [(520, 35000, 0), (300, 66000, 33024)])
-def test_wide_dh_units(T, V, vocab_group):
-    """A vocabulary group of at least 512 k-blocks that writes dH, with an even
-    number of column tiles in every sub-model, runs dH in wide units (two
-    column tiles sharing each A tile of G): widths of 2 and 4 column tiles (the
-    last ragged) over 3 or 2 token tiles (the last ragged).  In the second
-    case there are two groups of 33024 and 32976 columns: the first runs wide,
-    the second plain, accumulating into dH."""
-    wl = synth.Workload("wide", T=T, d=(320, 1008), V=V, tau=1.3, alpha=0.5, w_sigma=0.05)
+@pytest.mark.parametrize("T,V,vocab_group,ksplit", [(520, 35000, 0, [2]), (300, 66000, 33024, [3, 3])])
+def test_long_dh_reductions(T, V, vocab_group, ksplit):
+    """dH reductions of more than 512 k-blocks over 3 or 2 token tiles (the last
+    ragged) and 2 and 4 column tiles: too few tiles for the chip, so each
+    reduction is split over several units.  In the second case there are two
+    groups of 33024 and 32976 columns, the second adding its copies to dH."""
+    wl = synth.Workload("long", T=T, d=(320, 1008), V=V, tau=1.3, alpha=0.5, w_sigma=0.05)
+    assert launch_plan(wl, vocab_group)["ksplit"] == ksplit
     H, W, y = synth.make_inputs(wl, seed=13)
     full_parity(wl, H, W, y, vocab_group=vocab_group, argmax=False)
 
