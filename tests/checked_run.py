@@ -34,10 +34,13 @@ def main(path):
         out[f"dH{m}"] = op.dH[m].cpu().numpy()
         out[f"dW{m}"] = op.dW[m].cpu().numpy()
     # the backward GEMM's wide dH units (one group of 516 k-blocks, even
-    # column-tile counts), 8 partial states per token (two merge warps per 8
-    # tokens), and the pairwise metrics at M = 2 and M = 4 (their own tile
-    # widths)
-    for tag, wl2 in (("w", synth.Workload("chkw", T=1100, d=(320, 1008), V=33000, w_sigma=0.05)),
+    # column-tile counts), the same reductions split over several units, extra
+    # pairs in the head and evaluation launches, 8 partial states per token (two
+    # merge warps per 8 tokens), and the pairwise metrics at M = 2 and M = 4
+    # (their own tile widths)
+    for tag, wl2 in (("w", synth.Workload("chkw", T=2700, d=(264, 776), V=33000, w_sigma=0.05)),
+                     ("s", synth.Workload("chks", T=1100, d=(320, 1008), V=33000, w_sigma=0.05)),
+                     ("x", synth.Workload("chkx", T=1290, d=(72, 64, 80), V=25523, w_sigma=0.1)),
                      ("m4", synth.Workload("chk4", T=2048, d=(64, 128, 64, 192), V=2000, w_sigma=0.1))):
         H2, W2, y2 = synth.make_inputs(wl2, seed=75)
         H2, W2, y2 = [h.to(dev) for h in H2], [w.to(dev) for w in W2], y2.to(dev).to(torch.int32)
@@ -63,18 +66,21 @@ def main(path):
     torch.cuda.synchronize()
     out["status_junction"] = np.array(B.mls_get_status())
     out["jx"], out["jdo"], out["jde"] = (t.float().cpu().numpy() for t in (x, d_o, d_e))
-    # verify step, nucleus and greedy
-    sw = synth.SpecWorkload("chk", B=20, gamma=4, V=1500, d_draft=64, d_verify=128)
-    sd, swd, sv, swv = (t.to(dev) for t in synth.make_spec_inputs(sw, 73))
-    u = synth.make_uniforms(sw.B, sw.gamma, 73).to(dev)
-    draft = torch.randint(0, sw.V, (sw.B, sw.gamma), generator=torch.Generator().manual_seed(74),
-                          dtype=torch.int32).to(dev)
-    for greedy in (False, True):
-        sp = B.SpecVerify(sw.B, sw.gamma, sw.V, sw.d_draft, sw.d_verify, greedy=greedy, device=dev)
-        n, nx = sp(sd, swd, sv, swv, draft, u)
-        torch.cuda.synchronize()
-        out[f"status_spec{int(greedy)}"] = np.array(B.mls_get_status())
-        out[f"n{int(greedy)}"], out[f"next{int(greedy)}"] = n.cpu().numpy(), nx.cpu().numpy()
+    # verify step, nucleus and greedy: 150 rows (the pair GEMM's statistics
+    # epilogues), 100 rows (the few-row kernel, one tile per CTA), and 15 rows of
+    # 235 tiles in each head (several tiles of both heads per CTA)
+    for tag, sb, sV in (("a", 30, 1500), ("b", 20, 1500), ("c", 3, 30000)):
+        sw = synth.SpecWorkload("chk", B=sb, gamma=4, V=sV, d_draft=64, d_verify=128)
+        sd, swd, sv, swv = (t.to(dev) for t in synth.make_spec_inputs(sw, 73))
+        u = synth.make_uniforms(sw.B, sw.gamma, 73).to(dev)
+        draft = torch.randint(0, sw.V, (sw.B, sw.gamma), generator=torch.Generator().manual_seed(74),
+                              dtype=torch.int32).to(dev)
+        for greedy in (False, True):
+            sp = B.SpecVerify(sw.B, sw.gamma, sw.V, sw.d_draft, sw.d_verify, greedy=greedy, device=dev)
+            n, nx = sp(sd, swd, sv, swv, draft, u)
+            torch.cuda.synchronize()
+            out[f"status_spec{tag}{int(greedy)}"] = np.array(B.mls_get_status())
+            out[f"n{tag}{int(greedy)}"], out[f"next{tag}{int(greedy)}"] = n.cpu().numpy(), nx.cpu().numpy()
     np.savez(path, **out)
 
 
