@@ -10,7 +10,9 @@
 namespace mls {
 
 // Launches a kernel that may start before the stream's previous kernel has
-// completed (see chain_wait).
+// completed (see chain_wait).  An error goes to the caller only: unlike a plain
+// launch read with cudaGetLastError, cudaLaunchKernelEx would leave it behind as
+// the last error of the thread too.
 template <typename... P, typename... A>
 cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                            const A&... args) {
@@ -24,7 +26,9 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
   cfg.stream = s;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
 }
 
 constexpr int kMaxModels = 4;
@@ -177,10 +181,11 @@ struct GemmProblem {
   int tiles_n;                   // ceil(Ncols / kGemmBN)
   int tile_begin;                // first unit of this problem in the launch's unit numbering
                                  // (a unit is one pair tile of 256 x kGemmBN, or two if wide)
-  int tiles_m;                   // ceil(Mrows / 256); used when m_fast is set
+  int tiles_m;                   // ceil(Mrows / 256)
   int m_fast;                    // 1: consecutive tiles walk M first (pairs running at the
                                  //    same time share the B tile, read once from HBM)
-  // Epilogue (accumulate must be 0 unless kEpiPlain).  Per row and column tile
+  // Epilogue: kEpiPlain in launch_gemm_mixed, one of the others in
+  // launch_gemm_stats (accumulate 0).  Per row and column tile
   // (kGemmBN columns) the statistics go to stats[row * stats_ld + 2 * tile]:
   //   kEpiSoftmax: C = 2^((z - m_t) epi_scale), stats = (m_t, sum of C over the tile)
   //   kEpiArgmax:  C untouched, stats = (m_t, first column attaining m_t)
