@@ -129,10 +129,10 @@ __device__ __forceinline__ int fast_div(int n, const FastDiv& d) {
   return static_cast<int>((t + ((static_cast<unsigned>(n) - t) >> d.s1)) >> d.s2);
 }
 
-// A is MN-major for this problem.
+// A is MN-major for this problem (kAMode: 0 every A K-major, 2 per problem).
 template <int kAMode>
 __device__ __forceinline__ bool a_mn_of(const GemmProblem& pr) {
-  return kAMode == 2 ? pr.a_mn != 0 : kAMode == 1;
+  return kAMode == 2 && pr.a_mn != 0;
 }
 
 // Wide units exist only in the launch that mixes problems (launch_gemm_mixed).
@@ -472,9 +472,10 @@ __device__ __noinline__ void epilogue_stats(const GemmProblem& pr, const CUtenso
   }
 }
 
-// kStats: the launch may hold problems with a statistics epilogue (only the
-// verify step's logits GEMM); without it epilogue_stats is not in the kernel,
-// which keeps the training GEMMs at 64 registers instead of 119.
+// kStats: every problem has a statistics epilogue (the verify step's logits
+// GEMM, whose mapC is 2-D), otherwise every one has the plain epilogue (3-D
+// mapC); with both in one kernel the training GEMMs would take the statistics
+// epilogue's 118 registers instead of 80.
 template <int kAMode, bool kStats>
 __device__ __forceinline__ void gemm_epilogue(const GemmParams& p, uint32_t base, uint32_t tmem,
                                               uint32_t rank, int warp, int lane,
@@ -499,9 +500,8 @@ __device__ __forceinline__ void gemm_epilogue(const GemmParams& p, uint32_t base
         break;
       }
       tc_fence_after();
-      float v[32];
-      if (kStats && pr.epi != kEpiPlain) {
-        const int row0 = uc.tm * kPairM + static_cast<int>(rank) * kGemmBM + warp * 32;
+      const int row0 = uc.tm * kPairM + static_cast<int>(rank) * kGemmBM + warp * 32;
+      if constexpr (kStats) {
         const long long row = static_cast<long long>(row0) + lane;
         epilogue_stats(pr, &p.mapC[uc.prob], stage, stores, tl + acc * kGemmBN, tn, row,
                        row < pr.Mrows, row0, lane);
@@ -510,7 +510,7 @@ __device__ __forceinline__ void gemm_epilogue(const GemmParams& p, uint32_t base
         // stores (which drop what lies outside C), so that whole 128-byte lines
         // leave the SM.  One row per thread with 16-byte stores took about 13 us
         // per 256x256 tile, more than the MMAs of a tile with K < 2500.
-        const int row0 = uc.tm * kPairM + static_cast<int>(rank) * kGemmBM + warp * 32;
+        float v[32];
         const int ncols = row0 < pr.Mrows ? pr.Ncols - tn * kGemmBN : 0;
 #pragma unroll 1
         for (int c = 0; c * 32 < kGemmBN && c * 32 < ncols; ++c) {

@@ -7,8 +7,8 @@
 // (7 rows: as long as the reading itself).  So the operands change places: W's
 // vocabulary rows are the M dimension and the hidden rows the N dimension of
 // the MMA, whose time follows the rows there are.  One CTA per SM walks tiles
-// of 128 vocabulary columns over both sub-models' heads, with about 100 to 180
-// KB of W in flight per SM:
+// of 128 vocabulary columns over both sub-models' heads, with 96 to 160 KB of W
+// in flight per SM:
 //   warp 8    TMA producer: 128 rows of W and the n rows of H per k-block
 //   warp 9    MMA issuer
 //   warps 0-7 epilogue: one vocabulary column per lane, one MMA column per row

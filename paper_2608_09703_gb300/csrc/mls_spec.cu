@@ -98,42 +98,24 @@ __device__ __forceinline__ float comp(const float4& v, int j) {
 }
 
 // Block reductions: each warp reduces by a butterfly, lane 0 parks the
-// warp's partial, warp 0 combines the 16 partials by a butterfly and parks the
+// warp's partial, warp 0 combines the warps' partials by a butterfly and parks the
 // result for every thread.  Fixed order throughout.
-__device__ __forceinline__ void argmax_step(float& v, int& idx, float ov, int oi) {
-  if (ov > v || (ov == v && oi < idx)) {
-    v = ov;
-    idx = oi;
-  }
-}
-
-// (max value, lowest index attaining it).
 template <int NW>
-__device__ void block_argmax(float& v, int& idx, SharedT<NW>& sh) {
+__device__ float block_max(float v, SharedT<NW>& sh) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-    argmax_step(v, idx, __shfl_xor_sync(0xffffffffu, v, o), __shfl_xor_sync(0xffffffffu, idx, o));
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   __syncthreads();
-  if (lane_id() == 0) {
-    sh.f[warp_id()][0] = v;
-    sh.n[warp_id()][0] = idx;
-  }
+  if (lane_id() == 0) sh.f[warp_id()][0] = v;
   __syncthreads();
   if (warp_id() == 0) {
     const int l = lane_id();
-    float wv = l < NW ? sh.f[l][0] : -INFINITY;
-    int wi = l < NW ? sh.n[l][0] : 0x7fffffff;
+    float w = l < NW ? sh.f[l][0] : -INFINITY;
 #pragma unroll
-    for (int o = NW / 2; o > 0; o >>= 1)
-      argmax_step(wv, wi, __shfl_xor_sync(0xffffffffu, wv, o), __shfl_xor_sync(0xffffffffu, wi, o));
-    if (l == 0) {
-      sh.rf[0] = wv;
-      sh.rn[0] = wi;
-    }
+    for (int o = NW / 2; o > 0; o >>= 1) w = fmaxf(w, __shfl_xor_sync(0xffffffffu, w, o));
+    if (l == 0) sh.rf[0] = w;
   }
   __syncthreads();
-  v = sh.rf[0];
-  idx = sh.rn[0];
+  return sh.rf[0];
 }
 
 // Sums of a float and an int.
@@ -186,10 +168,9 @@ template <int NW>
 __device__ void row_stats(const float* st, int tiles, float scale, float* ftab, float* fg,
                           float& m, float& S, SharedT<NW>& sh) {
   float mv = -INFINITY;
-  int unused = 0;
   for (int t = threadIdx.x; t < tiles; t += NW * 32) mv = fmaxf(mv, st[2 * t]);
-  block_argmax(mv, unused, sh);
-  m = mv;
+  m = block_max(mv, sh);
+  int unused = 0;
   float s = 0.f;
   for (int t = threadIdx.x; t < tiles; t += NW * 32) {
     const float f = fast_exp2((st[2 * t] - m) * scale);
@@ -202,7 +183,7 @@ __device__ void row_stats(const float* st, int tiles, float scale, float* ftab, 
 }
 
 // Visits a row of unnormalised probabilities e[v] = e_t[v] f_t, warp w taking
-// the 128-element steps w, w + 16, ... (kUnroll of them per iteration):
+// the 128-element steps w, w + NW, ... (kUnroll of them per iteration):
 // `f(i0, e4, V)` gets the lane's 4 consecutive elements from index i0 (those
 // at or past V are not meaningful).  The loop is warp-uniform, so f may use
 // warp collectives.  Rows are 16-byte aligned and padded to 4 elements.
@@ -265,7 +246,7 @@ struct PassStats {
 };
 
 // One bisection pass over a whole row (e = e_t f_t), warps taking 128-token
-// steps w, w + 16, ..., kUnroll steps per iteration; only the row's last
+// steps w, w + NW, ..., kUnroll steps per iteration; only the row's last
 // float4 can be partial.
 template <bool kTrack, int NW>
 __device__ __forceinline__ void row_pass(const float* et, const float* ftab, int tsh, int V, uint32_t lo,
@@ -279,8 +260,7 @@ __device__ __forceinline__ void row_pass(const float* et, const float* ftab, int
       const int s0 = base + u * kStride, i0 = s0 + l * 4;
       // a tile whose maximum lies below the bracket holds no candidate
       const bool live = s0 < V && __float_as_uint(ftab[s0 >> tsh]) >= lo;
-      v[u] = live && i0 < V ? ld4(et + i0)
-                            : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[u] = live && i0 < V ? ld4(et + i0) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
@@ -904,9 +884,9 @@ __global__ void __launch_bounds__(NW * 32, 32 / NW) spec_row_kernel(const SpecPa
 
 // ------------------------------------------------------------------ sampling
 // Inverse-CDF sampling in index order over steps of 128 tokens: one pass gives
-// every step's mass (warps take steps w, w + 16, ...), one thread accumulates
-// them in index order, and one warp walks the step in which the cumulative
-// passes u * total.
+// every step's mass (two steps per warp and round), a block scan accumulates them
+// in index order, and one warp walks the step in which the cumulative passes
+// u * total.
 
 // Unnormalised probabilities e of the lane's 4 tokens from i0 (zeros past V).
 __device__ __forceinline__ float4 load_e(const float* et, const float* ftab, int tsh, long long i0,
@@ -1110,6 +1090,13 @@ __device__ int sample(const float* ep, const float* fp, const RowNucleus& np, co
   }
   __syncthreads();
   return sh.n[0][0];
+}
+
+__device__ __forceinline__ void argmax_step(float& v, int& idx, float ov, int oi) {
+  if (ov > v || (ov == v && oi < idx)) {
+    v = ov;
+    idx = oi;
+  }
 }
 
 // Greedy: the verifier's argmax of a row from its tile (max, argmax) pairs, by
