@@ -609,7 +609,9 @@ __device__ RowNucleus nucleus(const float* et, const float* st, float* fg, long 
   float mass_hi = 0.f, gt = 0.f;
   int eq = 0;
   bool resolved = false;
-  if (top_p < 1.f) {
+  // A NaN logit makes S and the target NaN, which no mass reaches: such a row
+  // keeps every token that is a number, as with top_p = 1.
+  if (top_p < 1.f && target == target) {
     const float* list = nullptr;  // candidates in shared memory, once they fit
     int n_list = 0;
     bool done = false;
