@@ -232,7 +232,13 @@ struct GemmCut {
 // in fp32 (6 dH tiles of 938 k-blocks) 261 against 73 us; 100 tokens, d =
 // (512, 1024), V = 20000 (6 of 313) 117 against 50 us; 20000 tokens, d =
 // (512, 1024), V = 600 (dW, 18 of 313) 117 against 78 us; 256 tokens, d = (128,
-// 256), V = 1024 in fp32 (2 of 32): a step of 55.9 against 53.1 us.
+// 256), V = 1024 in fp32 (2 of 32): a step of 55.9 against 53.1 us.  Where whole
+// reductions would run in wide units: 520 tokens, d = (320, 1008), V = 35000 317
+// against 112 us, 2000 tokens, d = (512, 1024), V = 50304 504 against 387 us.  At
+// the rule's far end, with 60 to 82 MB of copies: 7979 tokens, d = 416, V = 228345
+// 2266 against 2120 us; 8088, d = 504, V = 73613 779 against 768; 37116, d = (168,
+// 192), V = 49242 2480 against 2469; 7466 in fp32, d = 512, V = 192659 3974 against
+// 3944 us.
 constexpr int kSplitMinBlocks = 12, kSplitMost = 32;
 constexpr long long kSplitLaunch = 8, kSplitBytes = 1700000;
 constexpr double kSplitGain = 0.95;

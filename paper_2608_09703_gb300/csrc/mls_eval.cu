@@ -428,10 +428,10 @@ __device__ __forceinline__ bool eval_slots_main(const EvalParams& p, uint32_t ba
   for (int vt = tiles[0]; vt < tiles[1]; vt += tiles[2], ++j) {
     const uint32_t par = static_cast<uint32_t>(j) & 1u;
     const uint32_t sa = par * Sm::kN, sb = Sm::kN - sa;
-    // Column indices in 32 bits and one count of valid columns per tile: 64-bit
-    // comparisons per chunk cost the exposed pass 3 to 14% of the call (8192 tokens
-    // of the 3-level suite 3457 -> 3347 us; 54007 tokens, d = (216, 224, 2208), V =
-    // 20651: 5991 -> 5276 us).
+    // Column indices in 32 bits and one count of valid columns per tile, against
+    // 64-bit comparisons per chunk, which lengthen the exposed pass (whole calls, this
+    // step alone: 8192 tokens of the 3-level suite 3485 -> 3362 us; 54007 tokens,
+    // d = (216, 224, 2208), V = 20651: 6052 -> 5322 us).
     const int tcol = static_cast<int>(static_cast<unsigned>(vt) * Sm::kN + half * kHalf);
     const int left = static_cast<int>(min(static_cast<long long>(kHalf), p.V - static_cast<long long>(static_cast<unsigned>(tcol))));
     bool ok = mbar_wait(Sm::unit_full(base, 0), par, abort_flag, p.status);
@@ -631,10 +631,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kHeadThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   // The bounds of the tile loops stay in shared memory, read at every tile: the
-  // epilogue has no registers left for them.  8192 tokens of the 3-level suite
-  // took 3505 us per call with the bounds in registers, 3482 with them in the
-  // kernel's parameters (every pair alike) and 3337 this way; 4096 tokens of the
-  // 4-level suite 19.6, 19.8 and 18.4 ms.
+  // epilogue has no registers left for them.  This kernel with the split in a
+  // register and the rest in the parameters, against this: 8192 tokens of the
+  // 3-level suite 3594 -> 3335 us, 4096 tokens of the 4-level suite 20.4 -> 18.7
+  // ms, 2999 tokens of the pair d = (1024, 3072) 795 -> 716 us (interleaved calls
+  // whose spread is 5 to 15% under the power cap; timed tree after tree the 3-level
+  // call gained 4.6% with the merge below and the 32-bit columns above).
   volatile int* tiles = reinterpret_cast<volatile int*>(gbase + Sm::kTiles);
   int row_base;  // this CTA's tokens
   {
